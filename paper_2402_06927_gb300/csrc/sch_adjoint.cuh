@@ -400,6 +400,10 @@ __device__ __forceinline__ void backward_ck(const ModelArgs<R>& A, Shm<R, TP>* s
             load_field<R, C>(sl0 + A.n, st.u0);
             load_field<R, C>(sl1, st.m1);
             load_field<R, C>(sl1 + A.n, st.u1);
+            // the exchange below writes the slots hE, hF, which other warps may still be
+            // reading after the last barrier of a recomputed step or of the previous step's
+            // Matern solves
+            __syncthreads();
             chunk_halo2<R, C, TP>(st.m0, st.m0p, st.m0n, st.u0, st.u0p, st.u0n, sh);
             chunk_halo2<R, C, TP>(st.m1, st.m1p, st.m1n, st.u1, st.u1p, st.u1n, sh);
             R nq[C + 2];
