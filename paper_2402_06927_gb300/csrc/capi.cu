@@ -232,9 +232,32 @@ void cast_tab(const HTab& s, CTab<R>& d) {
     d.ge = (R)s.ge;
 }
 
+void fill_refine(const sch_params&, int, ModelArgs<float>&) {}
+void fill_refine(const sch_params& p, int C, ModelArgs<double>& A) {
+    const double h = p.L / p.n, g = 1.0 - 6.0 * p.alpha * p.alpha / (h * h);
+    HTab th;
+    RTab<double> q;
+    ctab_host(g, 6.0 - 2.0 * g, C, th);
+    cast_tab(th, A.helf);
+    rtab_host(th, p.n / C, q);
+    cast_rtab(q, A.rhelf);
+    A.helg = g;
+    A.c0f = (float)A.c0;
+    A.b0f = (float)A.b0;
+    A.tolf = (float)A.tol;
+    A.s6 = 3.0 / h;
+    A.kz = p.dt * h / 12.0;
+    for (int j = 0; j < p.K / 2; ++j)
+        for (int k = 0; k < 3; ++k) {
+            const double d = 2.0 * M_PI * (j + 1) * (k + 0.5) / p.n;
+            A.nco[j][k] = cos(d);
+            A.nsi[j][k] = sin(d);
+        }
+}
+
 template <typename R>
 void fill_args(const sch_params& p, int C, ModelArgs<R>& A) {
-    memset(&A, 0, sizeof(A));
+    memset(static_cast<void*>(&A), 0, sizeof(A));
     const double h = p.L / p.n;
     A.n = p.n;
     A.K = p.K;
@@ -299,6 +322,7 @@ void fill_args(const sch_params& p, int C, ModelArgs<R>& A) {
         A.mz = (R)(p.eta * sqrt(h) / 8.0);
         A.mk = p.matern_k;
     }
+    fill_refine(p, C, A);
 }
 
 // the warp-per-particle tables: sub-chunks of CS nodes, 64-row reduced systems

@@ -219,6 +219,230 @@ __device__ __forceinline__ void adjoint_step(const ModelArgs<R>& A, Shm<R, TP>* 
     chunk_halo<R, C, TP>(g, gp, gn, sh);
 }
 
+// FP64: the fixed point of adjoint_step by defect correction (the reasons and the float
+// solves are those of sch_refine.cuh).  Besides psi the iteration carries z, which
+// converges to H^{-1} B^T psi: with the current pair it forms in double
+//   r = g - P^T psi - (dt/2) M z,   then, psi updated, r' = B^T psi - H z,
+// and solves P^T for the change of psi and H for the change of z in float.  P^T is the
+// same in every iteration of a step, so its chunk sweep (q, al, ga), its interface rows
+// and warp 0's elimination of them are formed once a step and an iteration only runs
+// right-hand sides through them.  The float side is scaled by a power of two that takes
+// max|g| to [1, 2), so a gradient of any size stays in the float range; the stop test is
+// relative and does not see it.  14 FP64 instructions a node and iteration (about 45
+// before).  Returns false, with g unchanged, when the iteration does not converge or leaves
+// the float range: the caller then runs adjoint_step.
+template <int C, int TP>
+__device__ __forceinline__ bool adjoint_step_refined(const ModelArgs<double>& A, Shm<double, TP>* sh,
+                                                     const StepState<double, C>& st, const double (&nq)[C + 2],
+                                                     double (&g)[C], double& gp, double& gn, double (&gdu)[C],
+                                                     int& iters) {
+    const int t = threadIdx.x;
+    constexpr int NW = TP / 32;
+    // w = dv / 4 and S_i = mbar_i + mbar_{i+1} (S[0]: i = -1)
+    double w[C + 2], S[C + 1];
+    w[0] = A.dt8 * (st.u0p + st.u1p) + nq[0];
+    w[C + 1] = A.dt8 * (st.u0n + st.u1n) + nq[C + 1];
+#pragma unroll
+    for (int i = 0; i < C; ++i) w[i + 1] = A.dt8 * (st.u0[i] + st.u1[i]) + nq[i + 1];
+    {
+        double mb[C + 2];
+        mb[0] = st.m0p + st.m1p;
+        mb[C + 1] = st.m0n + st.m1n;
+#pragma unroll
+        for (int i = 0; i < C; ++i) mb[i + 1] = st.m0[i] + st.m1[i];
+#pragma unroll
+        for (int i = 0; i <= C; ++i) S[i] = 0.5 * (mb[i] + mb[i + 1]);
+    }
+    // the chunk sweep of P^T in float: rows (c0 + w_i, b0 + w_{i+1} - w_{i-1}, c0 - w_i)
+    float fa[C], fq[C], fal[C], fga[C], fc0, fqF;
+    {
+        float wf[C + 2], b[C], c[C];
+#pragma unroll
+        for (int i = 0; i < C + 2; ++i) wf[i] = d2f_bits(w[i]);
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            fa[i] = A.c0f + wf[i + 1];
+            c[i] = A.c0f - wf[i + 1];
+            b[i] = A.b0f + (wf[i + 2] - wf[i]);
+        }
+        fal[0] = -1.0f;
+        fga[0] = 0.0f;
+        fq[0] = 0.0f;
+#pragma unroll
+        for (int i = 1; i < C; ++i) {
+            fq[i] = rcp(b[i] - fa[i] * fga[i - 1]);
+            fga[i] = c[i] * fq[i];
+            fal[i] = -fa[i] * fal[i - 1] * fq[i];
+        }
+        fview(sh->ae)[t] = fal[C - 1];
+        fview(sh->ge)[t] = fga[C - 1];
+    }
+    // the forward coefficients ga (fgf) stay for the back sweep; al, ga become the back-swept weights
+    float fgf[C];
+    {
+        float ap = 0.0f, gpp = -1.0f;
+        fgf[0] = 0.0f;
+#pragma unroll
+        for (int i = 1; i < C; ++i) fgf[i] = fga[i];
+#pragma unroll
+        for (int i = C - 2; i >= 1; --i) {
+            ap = fal[i] - fgf[i] * ap;
+            gpp = -fgf[i] * gpp;
+            fal[i] = ap;
+            fga[i] = gpp;
+        }
+        fc0 = A.c0f - d2f_bits(w[1]);
+        fqF = rcp((A.b0f + (d2f_bits(w[2]) - d2f_bits(w[0]))) - fc0 * fal[1]);
+        fview(sh->pa)[t] = fa[0] * fqF;
+        fview(sh->pc)[t] = -fc0 * fga[1] * fqF;
+    }
+    // exponent of max|g| over the CTA: the scale of the float side
+    {
+        unsigned e = 0;
+#pragma unroll
+        for (int i = 0; i < C; ++i) e = max(e, (unsigned)__double2hiint(g[i]) & 0x7fffffffu);
+        e = __reduce_max_sync(FULL, e);
+        if ((t & 31) == 0) fview(sh->wred[0])[t >> 5] = __uint_as_float(e);
+    }
+    __syncthreads();
+    unsigned ge = 0;
+#pragma unroll
+    for (int r = 0; r < NW; ++r) ge = max(ge, __float_as_uint(fview(sh->wred[0])[r]));
+    ge >>= 20;
+    const int shq = min(1023 - (int)ge, 800) * (1 << 20);
+    int bad = ge >= 0x7ffu;
+    // warp 0: the elimination of the interface rows and the lane system's PCR multipliers
+    VarReduced<TP> V;
+    if (t < 32) V.factor(fview(sh->ae), fview(sh->ge), fview(sh->pa), fview(sh->pc), fview(sh->sw));
+    double psi[C], z[C], psip = 0.0, psin = 0.0, zp = 0.0, zn = 0.0;
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        psi[i] = 0.0;
+        z[i] = 0.0;
+    }
+    const double h2 = A.helg, kz = A.kz, s6 = A.s6;
+    int it = 1;
+    while (!bad) {
+        double lap[C];
+        float de[C], DF;
+        {
+            double dl = z[0] - zp;
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                const double dr = ((i == C - 1) ? zn : z[i + 1]) - z[i];
+                lap[i] = dr - dl;
+                dl = dr;
+            }
+            // r = g - P^T psi - (dt/2) (h/6) (6 z + second difference)
+            float d[C];
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                const double xl = (i == 0) ? psip : psi[i - 1], xr = (i == C - 1) ? psin : psi[i + 1];
+                double r = g[i] - A.c0 * (xl + xr);
+                r -= w[i + 1] * (xl - xr);
+                r -= (A.b0 + (w[i + 2] - w[i])) * psi[i];
+                r -= kz * (6.0 * z[i] + lap[i]);
+                d[i] = d2f_bits(r, shq);
+            }
+            de[0] = 0.0f;
+#pragma unroll
+            for (int i = 1; i < C; ++i) de[i] = (d[i] - fa[i] * de[i - 1]) * fq[i];
+            fview(sh->de)[t] = de[C - 1];
+            float dp = 0.0f;
+#pragma unroll
+            for (int i = C - 2; i >= 1; --i) {
+                dp = de[i] - fgf[i] * dp;
+                de[i] = dp;
+            }
+            DF = d[0] - fc0 * de[1];
+            fview(sh->pd)[t] = DF * fqF;
+        }
+        __syncthreads();                                             // B1
+        if (t < 32)
+            V.solve(fview(sh->ae), fview(sh->ge), fview(sh->pa), fview(sh->pc), fview(sh->pd), fview(sh->de),
+                    fview(sh->sw), fview(sh->E), fview(sh->F));
+        __syncthreads();                                             // B2
+        float dmax = 0.0f, pmax = 0.0f;
+        {
+            const float F = fview(sh->F)[t], E = fview(sh->E)[t];
+            psip += f2d_bits(fview(sh->E)[(t - 1) & (TP - 1)], shq);
+            psin += f2d_bits(fview(sh->F)[(t + 1) & (TP - 1)], shq);
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                const float dx = (i == 0) ? F : (i == C - 1) ? E : de[i] - fal[i] * F - fga[i] * E;
+                dmax = __uint_as_float(max(__float_as_uint(dmax), __float_as_uint(dx) & 0x7fffffffu));
+                psi[i] += f2d_bits(dx, shq);
+                pmax = __uint_as_float(max(__float_as_uint(pmax), __float_as_uint(d2f_bits(psi[i], shq)) & 0x7fffffffu));
+            }
+        }
+        dmax = warp_max_bits(dmax);
+        pmax = warp_max_bits(pmax);
+        if ((t & 31) == 0) {
+            fview(sh->wred[0])[t >> 5] = dmax;
+            fview(sh->wred[1])[t >> 5] = pmax;
+        }
+        // (6/h)(B^T psi - H z), (B^T x)_i = 1/2 (S_{i-1} x_{i-1} - S_i x_{i+1})
+        float dpH[C];
+        {
+            float r[C];
+#pragma unroll
+            for (int i = 0; i < C; ++i) {
+                const double xl = (i == 0) ? psip : psi[i - 1], xr = (i == C - 1) ? psin : psi[i + 1];
+                double e = s6 * (S[i] * xl - S[i + 1] * xr);
+                e -= 6.0 * z[i];
+                e -= h2 * lap[i];
+                r[i] = d2f_bits(e, shq);
+            }
+            helm_local_f<C, TP>(A.helf, r, dpH, sh);
+        }
+        __syncthreads();                                             // B3
+        if (t < 32) {
+            warp_solve_const<float, TP>(A.helf, A.rhelf, fview(sh->hpd), fview(sh->hde), fview(sh->hE), fview(sh->hF));
+            const float dm = warp_max_bits((t < NW) ? fview(sh->wred[0])[t] : 0.0f);
+            const float pm = warp_max_bits((t < NW) ? fview(sh->wred[1])[t] : 0.0f);
+            if (t == 0) {
+                int fl = 0;
+                if (!(dm < INFINITY) || !(pm < INFINITY)) fl = FLAG_NONFINITE;
+                else if (dm <= A.tolf * pm) fl = FLAG_CONVERGED;
+                sh->flag = fl;
+            }
+        }
+        __syncthreads();                                             // B4
+        {
+            const float hF = fview(sh->hF)[t], hE = fview(sh->hE)[t];
+            zp += f2d_bits(fview(sh->hE)[(t - 1) & (TP - 1)], shq);
+            zn += f2d_bits(fview(sh->hF)[(t + 1) & (TP - 1)], shq);
+            z[0] += f2d_bits(hF, shq);
+            z[C - 1] += f2d_bits(hE, shq);
+#pragma unroll
+            for (int i = 1; i < C - 1; ++i)
+                z[i] += f2d_bits(dpH[i] - A.helf.alpp[i] * hF - A.helf.gamp[i] * hE, shq);
+        }
+        const int fl = sh->flag;
+        if (fl & FLAG_CONVERGED) break;
+        bad = (fl & FLAG_NONFINITE) || it == A.max_iter;
+        ++it;
+    }
+    __syncthreads();   // the flag and the interface values are read
+    if (bad) return false;
+    iters += it;
+    // dJ/dm0 = N^T psi - (dt/2) M z, dJ/d(dU) = -B^T psi
+    double dl = z[0] - zp;
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        const double dr = ((i == C - 1) ? zn : z[i + 1]) - z[i];
+        const double xl = (i == 0) ? psip : psi[i - 1], xr = (i == C - 1) ? psin : psi[i + 1];
+        double r = A.c0p * (xl + xr) - w[i + 1] * (xl - xr);
+        r += (A.b0p - (w[i + 2] - w[i])) * psi[i];
+        r -= kz * (6.0 * z[i] + (dr - dl));
+        g[i] = r;
+        gdu[i] = 0.5 * (S[i + 1] * xr - S[i] * xl);
+        dl = dr;
+    }
+    chunk_halo<double, C, TP>(g, gp, gn, sh);
+    return true;
+}
+
 // sum over the CTA of sin(j theta_i) x_i and cos(j theta_i) x_i, j = 1 .. K/2:
 // each warp reduces with shuffles and lane 0 writes red[warp * K + 2(j-1) (+1)];
 // the caller sums over warps after a barrier.  (s1, c1): angle of node i0.
@@ -248,6 +472,51 @@ __device__ __forceinline__ void mode_sums_warp(const ModelArgs<R>& A, R s1, R c1
         cjm = cj;
         sj = sn2;
         cj = cn2;
+    }
+}
+
+// The same in FP64 for a four-node chunk about its centre theta_c: with x_{+-k} the values
+// at theta_c +- d_k, sum_k cos(j d_k) (x_k + x_-k) and sum_k sin(j d_k) (x_k - x_-k) carry
+// every harmonic, and four harmonics' eight sums cross the warp in one halving butterfly:
+// 13 FP64 instructions a harmonic and thread (38 before).
+__device__ __forceinline__ void mode_sums_centred(const ModelArgs<double>& A, double s1, double c1,
+                                                  const double (&x)[4], double* red) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double cd = A.nco[0][1], sd = A.nsi[0][1];
+    double sj = s1 * cd + c1 * sd, cj = c1 * cd - s1 * sd, sjm = 0.0, cjm = 1.0;
+    const double twoc = 2.0 * cj;
+    const double e0 = x[2] + x[1], o0 = x[2] - x[1], e1 = x[3] + x[0], o1 = x[3] - x[0];
+    for (int j0 = 0; j0 < A.K2; j0 += 4) {
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[2 * k] = 0.0;
+            v[2 * k + 1] = 0.0;
+            if (j0 + k < A.K2) {
+                const double E = A.nco[j0 + k][0] * e0 + A.nco[j0 + k][1] * e1;
+                const double O = A.nsi[j0 + k][0] * o0 + A.nsi[j0 + k][1] * o1;
+                v[2 * k] = sj * E + cj * O;
+                v[2 * k + 1] = cj * E - sj * O;
+                const double sn2 = twoc * sj - sjm, cn2 = twoc * cj - cjm;
+                sjm = sj;
+                cjm = cj;
+                sj = sn2;
+                cj = cn2;
+            }
+        }
+        // after the exchanges over 16, 8 and 4 a lane holds sum number (lane >> 2) of the eight
+#pragma unroll
+        for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1)
+#pragma unroll
+            for (int k = 0; k < h; ++k) {
+                const bool up = lane & o;
+                const double keep = up ? v[k + h] : v[k], send = up ? v[k] : v[k + h];
+                v[k] = keep + __shfl_xor_sync(FULL, send, o);
+            }
+        v[0] += __shfl_xor_sync(FULL, v[0], 2);
+        v[0] += __shfl_xor_sync(FULL, v[0], 1);
+        const int k = 2 * j0 + (lane >> 2);
+        if ((lane & 3) == 0 && k < A.K) red[warp * A.K + k] = v[0];
     }
 }
 
@@ -296,6 +565,74 @@ __device__ __forceinline__ void matern_adjoint_cells(const ModelArgs<R>& A, Shm<
     const R b = R(4) * A.mz;
 #pragma unroll
     for (int i = 0; i < C; ++i) gw[i] = b * (x[i] + ((i == C - 1) ? xn : x[i + 1]));
+}
+
+// The states (m, u) around step s, kept as four rows of n at sl, with chunk-end neighbours, and
+// the step's noise
+template <typename R, int C, int TP, int NZ>
+__device__ __forceinline__ void adjoint_load(const ModelArgs<R>& A, Shm<R, TP>* sh, const R* sl, R* noise,
+                                             const R* dW, const R* lam, int s, R s0, R c0, StepState<R, C>& st,
+                                             R (&nq)[C + 2]) {
+    load_field<R, C>(sl, st.m0);
+    load_field<R, C>(sl + A.n, st.u0);
+    load_field<R, C>(sl + 2 * A.n, st.m1);
+    load_field<R, C>(sl + 3 * A.n, st.u1);
+    // the exchange below writes the slots hE, hF, which other warps may still be
+    // reading after the last barrier of a recomputed step or of the previous step's
+    // Matern solves
+    __syncthreads();
+    chunk_halo2<R, C, TP>(st.m0, st.m0p, st.m0n, st.u0, st.u0p, st.u0n, sh);
+    chunk_halo2<R, C, TP>(st.m1, st.m1p, st.m1n, st.u1, st.u1p, st.u1n, sh);
+    if constexpr (NZ == SCH_NOISE_MATERN) {
+        matern_stage_step<R, C>(A, noise, dW, lam, s);
+        matern_nodes<R, C, TP>(A, sh, noise, nq);
+    } else if constexpr (sizeof(R) == 8) {
+        noise_nodes_centred(A, noise + s * A.K, s0, c0, nq);
+    } else {
+        noise_nodes<R, C>(A, noise + s * A.K, s0, c0, nq);
+    }
+}
+
+// adjoint_step of step s from its states
+template <typename R, int C, int TP, int NZ>
+__device__ __forceinline__ void adjoint_plain_body(const ModelArgs<R>& A, Shm<R, TP>* sh, const R* sl, R* noise,
+                                                   const R* dW, const R* lam, int s, R s0, R c0, R (&g)[C], R& gp,
+                                                   R& gn, R (&gdu)[C], int& iters, int& flags) {
+    StepState<R, C> st;
+    R nq[C + 2];
+    adjoint_load<R, C, TP, NZ>(A, sh, sl, noise, dW, lam, s, s0, c0, st, nq);
+    adjoint_step<R, C, TP>(A, sh, st, nq, g, gp, gn, gdu, iters, flags);
+}
+template <int C, int TP, int NZ>
+__device__ __noinline__ void adjoint_plain_f64(const ModelArgs<double>& A, Shm<double, TP>* sh, const double* sl,
+                                               double* noise, const double* dW, const double* lam, int s, double s0,
+                                               double c0, double (&g)[C], double& gp, double& gn, double (&gdu)[C],
+                                               int& iters, int& flags) {
+    adjoint_plain_body<double, C, TP, NZ>(A, sh, sl, noise, dW, lam, s, s0, c0, g, gp, gn, gdu, iters, flags);
+}
+template <typename R, int C, int TP, int NZ>
+__device__ __forceinline__ void adjoint_plain(const ModelArgs<R>& A, Shm<R, TP>* sh, const R* sl, R* noise,
+                                              const R* dW, const R* lam, int s, R s0, R c0, R (&g)[C], R& gp, R& gn,
+                                              R (&gdu)[C], int& iters, int& flags) {
+    if constexpr (sizeof(R) == 8) {
+        // out of line, on copies: only a step that adjoint_step_refined gives up comes here
+        R g2[C], d2[C], p2 = gp, q2 = gn;
+        int gi = 0, gf = 0;
+#pragma unroll
+        for (int i = 0; i < C; ++i) g2[i] = g[i];
+        adjoint_plain_f64<C, TP, NZ>(A, sh, sl, noise, dW, lam, s, s0, c0, g2, p2, q2, d2, gi, gf);
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            g[i] = g2[i];
+            gdu[i] = d2[i];
+        }
+        gp = p2;
+        gn = q2;
+        iters += gi;
+        flags |= gf;
+    } else {
+        adjoint_plain_body<R, C, TP, NZ>(A, sh, sl, noise, dW, lam, s, s0, c0, g, gp, gn, gdu, iters, flags);
+    }
 }
 
 // --------------------------------------------------------------------------
@@ -393,28 +730,16 @@ __device__ __forceinline__ void backward_ck(const ModelArgs<R>& A, Shm<R, TP>* s
             }
         }
         for (int s = sb - 1; s >= sa; --s) {
-            StepState<R, C> st;
-            const R* sl0 = seg + (size_t)(s - sa) * 2 * A.n;
-            const R* sl1 = sl0 + 2 * A.n;
-            load_field<R, C>(sl0, st.m0);
-            load_field<R, C>(sl0 + A.n, st.u0);
-            load_field<R, C>(sl1, st.m1);
-            load_field<R, C>(sl1 + A.n, st.u1);
-            // the exchange below writes the slots hE, hF, which other warps may still be
-            // reading after the last barrier of a recomputed step or of the previous step's
-            // Matern solves
-            __syncthreads();
-            chunk_halo2<R, C, TP>(st.m0, st.m0p, st.m0n, st.u0, st.u0p, st.u0n, sh);
-            chunk_halo2<R, C, TP>(st.m1, st.m1p, st.m1n, st.u1, st.u1p, st.u1n, sh);
-            R nq[C + 2];
-            if constexpr (NZ == SCH_NOISE_MATERN) {
-                matern_stage_step<R, C>(A, noise, dW, lam, s);
-                matern_nodes<R, C, TP>(A, sh, noise, nq);
-            } else {
-                noise_nodes<R, C>(A, noise + s * K, s0, c0, nq);
-            }
             R gdu[C];
-            adjoint_step<R, C, TP>(A, sh, st, nq, g, gp, gn, gdu, iters, flags);
+            bool done = false;
+            if constexpr (sizeof(R) == 8) {
+                StepState<R, C> st;
+                R nq[C + 2];
+                adjoint_load<R, C, TP, NZ>(A, sh, seg + (size_t)(s - sa) * 2 * A.n, noise, dW, lam, s, s0, c0, st, nq);
+                done = adjoint_step_refined<C, TP>(A, sh, st, nq, g, gp, gn, gdu, iters);
+            }
+            if (!done) adjoint_plain<R, C, TP, NZ>(A, sh, seg + (size_t)(s - sa) * 2 * A.n, noise, dW, lam, s, s0, c0,
+                                                   g, gp, gn, gdu, iters, flags);
             if constexpr (NZ == SCH_NOISE_MATERN) {
                 // one drift per cell: dJ/dlambda_c = dt dJ/dw_c + dt lambda_c, dJ/ddW_c = dJ/dw_c
                 R gw[C];
@@ -429,7 +754,10 @@ __device__ __forceinline__ void backward_ck(const ModelArgs<R>& A, Shm<R, TP>* s
                     }
                 }
             } else if (s >= v0 && s < v1) {
-                mode_sums_warp<R, C>(A, s1, c1, gdu, red);
+                if constexpr (sizeof(R) == 8)
+                    mode_sums_centred(A, s1, c1, gdu, red);
+                else
+                    mode_sums_warp<R, C>(A, s1, c1, gdu, red);
                 __syncthreads();
                 for (int k = t; k < K; k += TP) {
                     double sum = 0.0;

@@ -57,10 +57,25 @@ struct HBasis {
     R cpF, cpE, cpEp, cpFn, cdF, cdE, cdEp, cdFn;
 };
 
+// What the FP64 kernels' defect correction adds to ModelArgs (sch_refine.cuh): the float
+// tables of the correction solves and the noise tables about a four-node chunk's centre.
+template <typename R>
+struct RefineArgs {};
+template <>
+struct RefineArgs<double> {
+    CTab<float> helf;     // (6/h)(M + alpha^2 K)
+    RTab<float> rhelf;
+    double helg;          // its off-diagonal, 1 - 6 alpha^2 / h^2
+    float c0f, b0f, tolf;
+    double s6, kz;        // 3 / h, dt h / 12
+    // cos(j d_k), sin(j d_k) for harmonic j + 1 and offsets d_k = (k + 1/2) 2 pi / n
+    double nco[SCH_MAX_K / 2][3], nsi[SCH_MAX_K / 2][3];
+};
+
 // Precomputed scalars of the discretised model, passed by value to kernels
 // (so that every thread reads them from the constant parameter bank).
 template <typename R>
-struct ModelArgs {
+struct ModelArgs : RefineArgs<R> {
     int n, K, K2, M, stride, max_iter, solver;
     R h, dt;
     R c0, b0;      // left operator M + mu dt/2 K: off-diagonal, diagonal

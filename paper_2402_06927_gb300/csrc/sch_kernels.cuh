@@ -778,11 +778,19 @@ __device__ __forceinline__ void sch_step_ea(const ModelArgs<R>& A, Shm<R, TP>* s
     f.un = uin;
 }
 
+// FP64: the linearly implicit step by defect correction (sch_refine.cuh)
+template <int C, int TP, int NZ>
+__device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm<double, TP>* sh,
+                                                 Field<double, C>& f, const double* wq, double s0, double c0,
+                                                 int& iters, int& flags);
+
 template <int S, typename R, int C, int TP, int NZ = SCH_NOISE_MODES>
 __device__ __forceinline__ void step_any(const ModelArgs<R>& A, Shm<R, TP>* sh, Field<R, C>& f, const R* wq, R s0,
                                          R c0, int& iters, int& flags) {
     if constexpr (S == SCH_SOLVER_EA)
         sch_step_ea<R, C, TP, NZ>(A, sh, f, wq, s0, c0, iters, flags);
+    else if constexpr (sizeof(R) == 8)
+        sch_step_refined<C, TP, NZ>(A, sh, f, wq, s0, c0, iters, flags);
     else
         sch_step<R, C, TP, NZ>(A, sh, f, wq, s0, c0, iters, flags);
 }
@@ -1136,3 +1144,5 @@ struct Launch {
 };
 
 }  // namespace sch
+
+#include "sch_refine.cuh"
