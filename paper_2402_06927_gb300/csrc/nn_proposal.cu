@@ -15,48 +15,15 @@
 // operands to BF16 as it stages them in shared memory and accumulates in FP32
 // with mma.sync m16n8k16 (NN_BF16).  Parameters, activations and gradients stay
 // FP32 in memory in both (the FP32 master weights of Adam).
-#include <cuda_bf16.h>
-
-#include "sch_internal.h"
+#include "nn_internal.h"
 
 namespace sch {
-
-struct NNDims {
-    int n, K, Ns, C, M, prec;
-    float sigma;
-    int L[5];     // positions at layers 0..4: n, n/2, n/4, n/8, n/16
-    int cin[4];   // input channels of conv l
-    size_t off_w[4], off_b[4], off_wh, off_bh, nparam;
-    size_t act_off[5], off_F, off_lam, act_total;   // per-sample activation offsets (floats)
-};
-
-static NNDims make_dims(const nn_shape* s) {
-    NNDims d{};
-    d.n = s->n; d.K = s->K; d.Ns = s->Ns; d.C = s->C; d.M = s->M; d.sigma = s->sigma; d.prec = s->precision;
-    for (int l = 0; l <= 4; ++l) d.L[l] = s->n >> l;
-    size_t o = 0;
-    for (int l = 0; l < 4; ++l) {
-        d.cin[l] = (l == 0) ? 2 : s->C;
-        d.off_w[l] = o; o += (size_t)s->C * d.cin[l] * 5;
-        d.off_b[l] = o; o += (size_t)s->C;
-    }
-    d.off_wh = o; o += (size_t)s->K * s->Ns * s->C * s->K;
-    d.off_bh = o; o += (size_t)s->K * s->Ns;
-    d.nparam = o;
-    size_t a = 0;
-    d.act_off[0] = a; a += 2 * (size_t)d.L[0];
-    for (int l = 1; l <= 4; ++l) { d.act_off[l] = a; a += (size_t)s->C * d.L[l]; }
-    d.off_F = a; a += (size_t)s->C * s->K;
-    d.off_lam = a; a += (size_t)s->K * s->Ns;
-    d.act_total = a;
-    return d;
-}
 
 // --------------------------------------------------------------------------
 // tiled SGEMM: C[m][n] (+)= sum_k A(m, k) B(k, n) over a batch index z.
 // 64 x 64 tiles, k-chunks of 16, 256 threads, 4 x 4 outputs per thread.
 // --------------------------------------------------------------------------
-constexpr int TM = 64, TN = 64, TK = 16;
+constexpr int TK = 16;
 
 template <typename LA, typename LB, typename EP>
 __global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int Kd, int kchunk, LA la, LB lb, EP ep) {
@@ -132,14 +99,6 @@ struct is_transposed<F, decltype((void)F::transposed)> {
     static constexpr bool value = F::transposed;
 };
 
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
 template <typename LA, typename LB, typename EP>
 __global__ void __launch_bounds__(128) hgemm_kernel(int M, int N, int Kd, int kchunk, LA la, LB lb, EP ep) {
     __shared__ __align__(16) __nv_bfloat16 As[HTM][HTK + HPAD];   // [m][k]
@@ -208,19 +167,6 @@ __global__ void __launch_bounds__(128) hgemm_kernel(int M, int N, int Kd, int kc
                 const int gn = n0 + wn + 8 * j + 2 * tq + (e & 1);
                 if (gm < M && gn < N) ep(zb, gm, gn, acc[i][j][e]);
             }
-}
-
-// k-splits for a reduction with few output tiles (weight gradients: the sum runs over
-// batch x positions): about 8 CTAs per SM, chunks of at least 256 k-values
-static int splitk_for(int M, int N, int Kd) {
-    const int tiles = ((M + TM - 1) / TM) * ((N + TN - 1) / TN);
-    return max(1, min(Kd / 256, 8 * device_sms() / tiles));
-}
-
-// k-chunks that sgemm launches for a split of splitk
-static int splitk_chunks(int Kd, int splitk) {
-    const int kchunk = (Kd + splitk - 1) / splitk;
-    return (Kd + kchunk - 1) / kchunk;
 }
 
 // the GEMM in the network's precision: the FP32 SIMT kernel or the BF16 tensor-core kernel
@@ -592,23 +538,6 @@ __global__ void __launch_bounds__(128) conv0_cl_kernel(int n, int M, float sigma
     cl_store_tile(Os, out + (size_t)b * out_bs + (size_t)q0 * CL_C);
 }
 
-// 16-byte asynchronous copy global -> shared (cp.async, completion tracked by groups)
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-
-// four 8 x 8 BF16 matrices from shared memory (lane l gives the address of row l % 8 of
-// matrix l / 8); register i receives matrix i in the mma fragment layout
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const void* smem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(sa));
-}
-
 // The input slab of tile (b, q0): positions 2 q0 - 2 + r, r = 0 .. 130 (mod Lin), 64 channels
 // each, stored de-interleaved: offset r at row r / 2 when r is even, CL_XEVEN + r / 2 when odd,
 // so that the rows 2q + j of the output positions q of a fragment are consecutive.
@@ -884,8 +813,9 @@ size_t nn_workspace_bytes(const nn_shape* s, int B) {
     if (!s || B <= 0 || nn_param_count(s) == 0) return 0;
     const NNDims d = make_dims(s);
     // forward activations + two gradient buffers of one activation each + glam/gF + split-K partials
-    return ((size_t)B * d.act_total * 3 + 2 * (size_t)d.C * d.K * B + (size_t)d.K * d.Ns * B +
-            partial_floats(d, B)) * sizeof(float);
+    const size_t generic = ((size_t)B * d.act_total * 3 + 2 * (size_t)d.C * d.K * B + (size_t)d.K * d.Ns * B +
+                            partial_floats(d, B)) * sizeof(float);
+    return cf_supported(d) ? max(generic, cf_workspace_bytes(d, B)) : generic;
 }
 
 static int nn_check(const nn_shape* s, int B, const void* params, const void* u, const void* y, void* ws,
@@ -921,6 +851,8 @@ int nn_backward(const nn_shape* s, int B, const float* params, const float* u_st
     if (!target || !grads || !loss || y_stride < 0) return SCH_ERR_ARG;
     const NNDims d = make_dims(s);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (cf_supported(d) && (size_t)B * d.n < (1u << 31))
+        return nn_backward_cf(d, B, params, u_start, y, y_stride, target, grads, loss, ws, st);
     float* act = reinterpret_cast<float*>(ws);
     const size_t bs = d.act_total;
     float* gA = act + (size_t)B * bs;          // gradient of an activation (ping)
