@@ -79,6 +79,20 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const void* smem) 
                  : "r"(sa));
 }
 
+// the same, each matrix transposed
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], const void* smem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(sa));
+}
+
+// nn_forward with NN_BF16 on channels-last BF16 activations (nn_infer.cu)
+bool cl_supported(const NNDims& d);
+size_t cl_workspace_bytes(const NNDims& d, int B);
+int nn_forward_cl(const NNDims& d, int B, const float* params, const float* u, const float* y, int ystride, void* ws,
+                  float* lam_out, cudaStream_t st);
+
 // nn_backward with NN_BF16 on channels-first BF16 activations (nn_train.cu): whether a shape
 // takes it, its workspace bytes, and the pass itself (loss and every gradient)
 bool cf_supported(const NNDims& d);

@@ -286,13 +286,6 @@ struct Store {            // out[z * bs + m * ld + n] = v (+ bias[n] if bias)
         out[(size_t)z * bs + (size_t)m * ld + n] = v + (bias ? bias[n] : 0.f);
     }
 };
-struct StoreBF16 {        // out[z * bs + m * ld + n] = v rounded to BF16
-    __nv_bfloat16* out; size_t bs; int ld;
-    __device__ void operator()(int z, int m, int n, float v) const {
-        out[(size_t)z * bs + (size_t)m * ld + n] = __float2bfloat16_rn(v);
-    }
-};
-
 // --------------------------------------------------------------------------
 // element-wise kernels
 // --------------------------------------------------------------------------
@@ -419,373 +412,6 @@ static void nn_forward_impl(const NNDims& d, int B, const float* params, const f
           Store{act + d.off_lam, 0, (int)bs, params + d.off_bh}, st);
 }
 
-// --------------------------------------------------------------------------
-// BF16 inference path with channels-last activations (nn_forward with NN_BF16 and
-// C = 64): the activations of layers 1..4 are stored once as BF16, [b][position][c],
-// so that a convolution's operand pairs (channel ci, ci + 1 at one input position)
-// are adjacent and a tile's im2col is the input slab itself.  Layer 0 (two input
-// channels, 10 taps) runs on the CUDA cores from the features; layers 1..3 on the
-// tensor cores (conv_tc_kernel); the mode projection and the head through
-// hgemm_kernel.  Values equal the BF16 path of nn_forward_impl (the same BF16
-// rounding of every operand), accumulation orders aside.
-// --------------------------------------------------------------------------
-constexpr int CL_C = 64;                 // channels of the channels-last path
-constexpr int CL_K = 5 * CL_C;           // reduction length of layers 1..3 (k = j C + ci)
-constexpr int CL_WROW = CL_K + 8;        // shared weight row (bf16): 656 bytes, 16 mod 128
-constexpr int CL_XROW = CL_C + 8;        // shared slab row (bf16): 144 bytes, 16 mod 128
-constexpr int CL_TQ = 64;                // output positions per CTA
-constexpr int CL_XPOS = 2 * CL_TQ + 3;   // input positions a tile reads
-constexpr int CL_XEVEN = CL_TQ + 2;      // of which at even offsets from the slab's start
-
-__host__ __device__ constexpr size_t cl_smem() {
-    return ((size_t)CL_C * CL_WROW + 2 * (size_t)CL_XPOS * CL_XROW + (size_t)CL_TQ * (CL_C + 8)) *
-           sizeof(__nv_bfloat16);
-}
-
-// the weights of conv layers 1..3 as BF16 [l][co][j C + ci] (k ordered tap-major)
-__global__ void pack_conv_weights_kernel(const float* params, size_t off1, size_t off2, size_t off3,
-                                         __nv_bfloat16* wb) {
-    const int tot = 3 * CL_C * CL_K;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += gridDim.x * blockDim.x) {
-        const int l = e / (CL_C * CL_K), r = e % (CL_C * CL_K);
-        const int co = r / CL_K, k = r % CL_K, j = k / CL_C, ci = k % CL_C;
-        const size_t off = (l == 0) ? off1 : (l == 1) ? off2 : off3;
-        wb[e] = __float2bfloat16_rn(params[off + ((size_t)co * CL_C + ci) * 5 + j]);
-    }
-}
-
-// Layer 0 on the tensor cores: out[b][q][co] = relu(b0[co] + sum_k X0[q][k] W0[co][k]) with
-// k = 2 j + ci (ten taps x channels, padded to 16 with zero weights), X0[q][k] the feature
-// of channel ci at input position 2q + j - 2.  A CTA takes 64 output positions of one
-// sample: its threads form the features of the positions 2 q0 - 2 .. 2 q0 + 133 as BF16
-// (u, innovation) pairs in shared memory, so that row q of X0 is 16 consecutive values
-// starting at pair 2q; warp w then computes the 32 x 32 quarter (w / 2, w % 2) of the
-// 64 x 64 output with one k-step of mma.sync m16n8k16.  Epilogue: bias, ReLU, BF16, the
-// tile staged in shared memory and stored as 8 KB of contiguous rows.
-constexpr int CL_OROW = CL_C + 8;         // staged output row (bf16): 144 bytes, rows in distinct banks
-
-// a CTA's 64 x 64 output tile, staged in shared memory [64][CL_OROW], to the 64 consecutive
-// channels-last rows from dst (8 KB contiguous): 16-byte stores, 128 threads
-__device__ __forceinline__ void cl_store_tile(const __nv_bfloat16* Os, __nv_bfloat16* dst) {
-    for (int e = threadIdx.x; e < 64 * (CL_C / 8); e += 128) {
-        const int r = e / (CL_C / 8), c8 = e % (CL_C / 8);
-        *reinterpret_cast<uint4*>(dst + (size_t)r * CL_C + 8 * c8) =
-            *reinterpret_cast<const uint4*>(Os + r * CL_OROW + 8 * c8);
-    }
-}
-
-constexpr int C0_TQ = 64;                 // output positions per CTA
-constexpr int C0_XPOS = 2 * C0_TQ + 8;    // feature positions staged (rows read 8 positions)
-constexpr int C0_WROW = 16 + 8;           // shared weight row (bf16)
-
-__global__ void __launch_bounds__(128) conv0_cl_kernel(int n, int M, float sigma, const float* u, const float* y,
-                                                       int ystride, const float* w0, const float* b0,
-                                                       __nv_bfloat16* out, size_t out_bs) {
-    __shared__ __align__(16) __nv_bfloat16 Xs[2 * C0_XPOS];      // (u, innovation) per position
-    __shared__ __align__(16) __nv_bfloat16 Ws[CL_C * C0_WROW];   // [co][2 j + ci], zero for k >= 10
-    __shared__ __align__(16) __nv_bfloat16 Os[C0_TQ * CL_OROW];  // the output tile
-    const int b = blockIdx.y, q0 = blockIdx.x * C0_TQ, stride = n / M;
-    for (int e = threadIdx.x; e < CL_C * 16; e += 128) {
-        const int co = e / 16, k = e % 16, j = k >> 1, ci = k & 1;
-        Ws[co * C0_WROW + k] = __float2bfloat16_rn(k < 10 ? w0[(co * 2 + ci) * 5 + j] : 0.f);
-    }
-    for (int r = threadIdx.x; r < C0_XPOS; r += 128) {
-        const int i = (2 * q0 - 2 + r + n) % n;
-        const float ub = u[(size_t)b * n + i];
-        float inn = 0.f;
-        if (i % stride == 0) {
-            const float yj = y[(size_t)b * ystride + i / stride];
-            if (yj == yj) inn = (yj - ub) / sigma;   // NaN: not observed
-        }
-        *reinterpret_cast<__nv_bfloat162*>(Xs + 2 * r) = __floats2bfloat162_rn(ub, inn);
-    }
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wq = (warp >> 1) * 32, wc = (warp & 1) * 32;
-    const int gq = lane >> 2, tq = lane & 3;
-    uint32_t a[2][4], bf[4][2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int q = wq + 16 * i + gq;   // row q starts at pair 2q; k pair (2t, 2t+1) is pair 2q + t
-        a[i][0] = *reinterpret_cast<const uint32_t*>(Xs + 2 * (2 * q + tq));
-        a[i][1] = *reinterpret_cast<const uint32_t*>(Xs + 2 * (2 * (q + 8) + tq));
-        a[i][2] = *reinterpret_cast<const uint32_t*>(Xs + 2 * (2 * q + tq + 4));
-        a[i][3] = *reinterpret_cast<const uint32_t*>(Xs + 2 * (2 * (q + 8) + tq + 4));
-    }
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-        const int c = wc + 8 * jj + gq;
-        bf[jj][0] = *reinterpret_cast<const uint32_t*>(Ws + c * C0_WROW + 2 * tq);
-        bf[jj][1] = *reinterpret_cast<const uint32_t*>(Ws + c * C0_WROW + 2 * tq + 8);
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};
-            mma_bf16_16816(acc, a[i], bf[jj]);
-            const int co = wc + 8 * jj + 2 * tq;
-            const float bb0 = b0[co], bb1 = b0[co + 1];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int q = wq + 16 * i + gq + 8 * h;
-                const float v0 = acc[2 * h] + bb0, v1 = acc[2 * h + 1] + bb1;
-                *reinterpret_cast<__nv_bfloat162*>(Os + q * CL_OROW + co) =
-                    __floats2bfloat162_rn(v0 > 0.f ? v0 : 0.f, v1 > 0.f ? v1 : 0.f);
-            }
-        }
-    __syncthreads();
-    cl_store_tile(Os, out + (size_t)b * out_bs + (size_t)q0 * CL_C);
-}
-
-// The input slab of tile (b, q0): positions 2 q0 - 2 + r, r = 0 .. 130 (mod Lin), 64 channels
-// each, stored de-interleaved: offset r at row r / 2 when r is even, CL_XEVEN + r / 2 when odd,
-// so that the rows 2q + j of the output positions q of a fragment are consecutive.
-__device__ __forceinline__ int cl_slab_row(int r) { return (r & 1) ? CL_XEVEN + (r >> 1) : (r >> 1); }
-
-__device__ __forceinline__ void cl_issue_slab(__nv_bfloat16* Xs, const __nv_bfloat16* in, size_t in_bs, int Lin,
-                                              int b, int q0) {
-    const __nv_bfloat16* inb = in + (size_t)b * in_bs;
-    for (int e = threadIdx.x; e < CL_XPOS * (CL_C / 8); e += 128) {
-        const int r = e / (CL_C / 8), c8 = e % (CL_C / 8);
-        const int pos = (2 * q0 - 2 + r + Lin) % Lin;
-        cp_async16(Xs + cl_slab_row(r) * CL_XROW + 8 * c8, inb + (size_t)pos * CL_C + 8 * c8);
-    }
-}
-
-// Layers 1..3 on the tensor cores: D[q][co] = sum_k X[q][k] W[co][k], k = j C + ci and
-// X[q][k] = in[b][(2q + j - 2) mod Lin][ci].  A persistent CTA stages the layer's weights
-// [64][320] in shared memory once, then takes tiles of 64 output positions of one sample
-// (all 64 output channels) in turn: the input slab of positions 2 q0 - 2 .. 2 q0 + 128
-// (131 rows of 64 channels) is copied with cp.async into one of two buffers while the
-// previous tile is computed.  Warp w computes the 32 x 32 quarter (w / 2, w % 2) of a
-// tile with mma.sync m16n8k16, its A fragments loaded by ldmatrix straight from the slab
-// (rows 2q + j, 16 channels), its B fragments from the weights.  Epilogue: bias, ReLU,
-// BF16, the tile staged in shared memory and stored as 8 KB of contiguous rows.
-__global__ void __launch_bounds__(128) conv_tc_kernel(int B, int Lin, const __nv_bfloat16* __restrict__ in,
-                                                      size_t in_bs, const __nv_bfloat16* __restrict__ wb,
-                                                      const float* __restrict__ bias, __nv_bfloat16* __restrict__ out,
-                                                      size_t out_bs) {
-    extern __shared__ __align__(16) unsigned char cl_raw[];
-    __nv_bfloat16* Ws = reinterpret_cast<__nv_bfloat16*>(cl_raw);   // [64][CL_WROW]
-    __nv_bfloat16* Xbuf = Ws + CL_C * CL_WROW;                       // [2][CL_XPOS][CL_XROW]
-    __nv_bfloat16* Os = Xbuf + 2 * CL_XPOS * CL_XROW;                // [CL_TQ][CL_OROW] output tile
-    const int tpb = (Lin / 2) / CL_TQ, ntiles = B * tpb;
-    for (int e = threadIdx.x; e < CL_C * (CL_K / 8); e += 128) {
-        const int r = e / (CL_K / 8), c8 = e % (CL_K / 8);
-        *reinterpret_cast<uint4*>(Ws + r * CL_WROW + 8 * c8) = *reinterpret_cast<const uint4*>(wb + r * CL_K + 8 * c8);
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // the rows and column halves this lane addresses in ldmatrix: A (slab) matrices are
-    // (rows 0-7, 8-15) x (columns 0-7, 8-15), B (weight) matrices (k 0-7, 8-15) x (n 0-7, 8-15)
-    const int arow = (lane & 7) + 8 * ((lane >> 3) & 1), acol = 8 * (lane >> 4);
-    const int brow = (lane & 7) + 8 * (lane >> 4), bcol = 8 * ((lane >> 3) & 1);
-    const int wq = (warp >> 1) * 32, wc = (warp & 1) * 32;
-    const int gq = lane >> 2, tq = lane & 3;
-    int t = blockIdx.x;
-    if (t < ntiles) cl_issue_slab(Xbuf, in, in_bs, Lin, t / tpb, (t % tpb) * CL_TQ);
-    cp_async_commit();
-    for (int it = 0; t < ntiles; t += gridDim.x, ++it) {
-        const int tn = t + gridDim.x;
-        if (tn < ntiles)
-            cl_issue_slab(Xbuf + ((it + 1) & 1) * CL_XPOS * CL_XROW, in, in_bs, Lin, tn / tpb, (tn % tpb) * CL_TQ);
-        cp_async_commit();
-        cp_async_wait1();   // this tile's slab (the group before the one just committed)
-        __syncthreads();
-        const __nv_bfloat16* Xs = Xbuf + (it & 1) * CL_XPOS * CL_XROW;
-        const int b = t / tpb, q0 = (t % tpb) * CL_TQ;
-        float acc[2][4][4];
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) acc[i][jj][e] = 0.f;
-#pragma unroll 1
-        for (int j = 0; j < 5; ++j) {
-            // slab rows of tap j: offset 2q + j is row q + j/2 (even j) or CL_XEVEN + q + (j-1)/2
-            const int jrow = (j & 1) ? CL_XEVEN + (j >> 1) : (j >> 1);
-#pragma unroll
-            for (int kc = 0; kc < CL_C; kc += 16) {
-                uint32_t a[2][4], bf[4][2];
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    ldmatrix_x4(a[i], Xs + (jrow + wq + 16 * i + arow) * CL_XROW + kc + acol);
-#pragma unroll
-                for (int jj = 0; jj < 4; jj += 2) {
-                    uint32_t r4[4];
-                    ldmatrix_x4(r4, Ws + (wc + 8 * jj + brow) * CL_WROW + j * CL_C + kc + bcol);
-                    bf[jj][0] = r4[0];
-                    bf[jj][1] = r4[1];
-                    bf[jj + 1][0] = r4[2];
-                    bf[jj + 1][1] = r4[3];
-                }
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) mma_bf16_16816(acc[i][jj], a[i], bf[jj]);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-                const int co = wc + 8 * jj + 2 * tq;
-                const float b0 = bias[co], b1 = bias[co + 1];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int q = wq + 16 * i + gq + 8 * h;
-                    const float v0 = acc[i][jj][2 * h] + b0, v1 = acc[i][jj][2 * h + 1] + b1;
-                    const __nv_bfloat162 pk = __floats2bfloat162_rn(v0 > 0.f ? v0 : 0.f, v1 > 0.f ? v1 : 0.f);
-                    *reinterpret_cast<__nv_bfloat162*>(Os + q * CL_OROW + co) = pk;
-                }
-            }
-        __syncthreads();
-        cl_store_tile(Os, out + (size_t)b * out_bs + (size_t)q0 * CL_C);
-        __syncthreads();   // every warp is done with this buffer and the output tile before reuse
-    }
-}
-
-// BF16 weights of the head, Wh [K Ns][C K] in the parameters' layout
-__global__ void pack_bf16_kernel(size_t count, const float* src, __nv_bfloat16* dst) {
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x)
-        dst[e] = __float2bfloat16_rn(src[e]);
-}
-
-// Dense GEMM with BF16 operands from memory and FP32 accumulation (the head of the
-// channels-last path): C[m][n] = sum_k A[m][k] B[n][k] + bias[n], A [M][Kd] and B [N][Kd]
-// row-major BF16, Kd a multiple of 32.  64 x 64 tiles, 128 threads (warp w: the 32 x 32
-// quarter (w / 2, w % 2)), k-chunks of 32 double-buffered with cp.async, fragments by
-// ldmatrix (80-byte shared rows: eight rows fall in distinct 16-byte bank groups).
-constexpr int DG_T = 64, DG_BK = 32, DG_ROW = DG_BK + 8;
-
-__global__ void __launch_bounds__(128) dense_bf16_gemm_kernel(int M, int N, int Kd,
-                                                              const __nv_bfloat16* __restrict__ A,
-                                                              const __nv_bfloat16* __restrict__ Bm,
-                                                              const float* __restrict__ bias, float* __restrict__ C,
-                                                              int ldc) {
-    __shared__ __align__(16) __nv_bfloat16 As[2][DG_T][DG_ROW];
-    __shared__ __align__(16) __nv_bfloat16 Bs[2][DG_T][DG_ROW];
-    const int m0 = blockIdx.y * DG_T, n0 = blockIdx.x * DG_T;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    const int gq = lane >> 2, tq = lane & 3;
-    const int arow = (lane & 7) + 8 * ((lane >> 3) & 1), acol = 8 * (lane >> 4);
-    const int brow = (lane & 7) + 8 * (lane >> 4), bcol = 8 * ((lane >> 3) & 1);
-    auto issue = [&](int buf, int k0) {
-        for (int e = threadIdx.x; e < DG_T * (DG_BK / 8); e += 128) {
-            const int r = e / (DG_BK / 8), c8 = e % (DG_BK / 8);
-            const int gm = min(m0 + r, M - 1), gn = min(n0 + r, N - 1);   // rows past the end: any row
-            cp_async16(&As[buf][r][8 * c8], A + (size_t)gm * Kd + k0 + 8 * c8);
-            cp_async16(&Bs[buf][r][8 * c8], Bm + (size_t)gn * Kd + k0 + 8 * c8);
-        }
-    };
-    float acc[2][4][4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[i][jj][e] = 0.f;
-    const int nk = Kd / DG_BK;
-    issue(0, 0);
-    cp_async_commit();
-    for (int kt = 0; kt < nk; ++kt) {
-        if (kt + 1 < nk) issue((kt + 1) & 1, (kt + 1) * DG_BK);
-        cp_async_commit();
-        cp_async_wait1();
-        __syncthreads();
-        const int b = kt & 1;
-#pragma unroll
-        for (int ks = 0; ks < DG_BK; ks += 16) {
-            uint32_t a[2][4], bf[4][2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) ldmatrix_x4(a[i], &As[b][wm + 16 * i + arow][ks + acol]);
-#pragma unroll
-            for (int jj = 0; jj < 4; jj += 2) {
-                uint32_t r4[4];
-                ldmatrix_x4(r4, &Bs[b][wn + 8 * jj + brow][ks + bcol]);
-                bf[jj][0] = r4[0];
-                bf[jj][1] = r4[1];
-                bf[jj + 1][0] = r4[2];
-                bf[jj + 1][1] = r4[3];
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int jj = 0; jj < 4; ++jj) mma_bf16_16816(acc[i][jj], a[i], bf[jj]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int gm = m0 + wm + 16 * i + gq + ((e & 2) ? 8 : 0);
-                const int gn = n0 + wn + 8 * jj + 2 * tq + (e & 1);
-                if (gm < M && gn < N) C[(size_t)gm * ldc + gn] = acc[i][jj][e] + bias[gn];
-            }
-}
-
-// A(c, q) = h[b][q][c] of a channels-last BF16 activation (the mode projection's operand)
-struct CLRows {
-    static constexpr bool transposed = true;
-    const __nv_bfloat16* h; size_t bstride;
-    __device__ float operator()(int b, int m, int k) const {
-        return __bfloat162float(h[(size_t)b * bstride + (size_t)k * CL_C + m]);
-    }
-};
-
-// bytes of the channels-last inference path's buffers per sample: layers 1..4 in BF16,
-// the mode features F and lambda in FP32 (together below the FP32 path's act_total floats)
-static size_t cl_act_elems(const NNDims& d) {
-    return (size_t)CL_C * (d.L[1] + d.L[2] + d.L[3] + d.L[4]);
-}
-
-static bool cl_supported(const NNDims& d) {
-    // 64 channels; every layer's output a whole number of 64-position tiles; the head's
-    // reduction C K a multiple of the dense GEMM's k-chunk
-    return d.prec == NN_BF16 && d.C == CL_C && d.L[4] % CL_TQ == 0 && (d.C * d.K) % DG_BK == 0;
-}
-
-static void nn_forward_cl(const NNDims& d, int B, const float* params, const float* u, const float* y, int ystride,
-                          void* ws, float* lam_out, cudaStream_t st) {
-    const size_t cs = cl_act_elems(d);
-    __nv_bfloat16* act = reinterpret_cast<__nv_bfloat16*>(ws);
-    const int P = d.L[4], FF = d.C * d.K, O = d.K * d.Ns;
-    __nv_bfloat16* wb = act + (size_t)B * cs;                               // [3][64][320]
-    __nv_bfloat16* whb = wb + 3 * CL_C * CL_K;                              // [O][FF]
-    __nv_bfloat16* F = whb + (size_t)O * FF;                                // [B][C K]
-    size_t off[5];
-    off[1] = 0;
-    for (int l = 1; l < 4; ++l) off[l + 1] = off[l] + (size_t)CL_C * d.L[l];
-    pack_conv_weights_kernel<<<grid_elems(3 * CL_C * CL_K), 256, 0, st>>>(params, d.off_w[1], d.off_w[2], d.off_w[3],
-                                                                           wb);
-    conv0_cl_kernel<<<dim3(d.L[1] / C0_TQ, B), 128, 0, st>>>(d.n, d.M, d.sigma, u, y, ystride, params + d.off_w[0],
-                                                            params + d.off_b[0], act + off[1], cs);
-    const size_t sm = cl_smem();
-    cudaFuncSetAttribute(conv_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    // persistent CTAs: as many as fit on the device at once (two per SM at 78 KB of shared memory)
-    int dev = 0, nsm = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, conv_tc_kernel, 128, sm);
-    const int resident = max(1, nsm * max(1, per_sm));
-    for (int l = 1; l < 4; ++l) {
-        const int ntiles = B * (d.L[l + 1] / CL_TQ);
-        conv_tc_kernel<<<min(ntiles, resident), 128, sm, st>>>(B, d.L[l], act + off[l], cs,
-                                                               wb + (size_t)(l - 1) * CL_C * CL_K, params + d.off_b[l],
-                                                               act + off[l + 1], cs);
-    }
-    // F = h4 S / P in BF16 (the head's operand), then lambda = F Wh^T + bh
-    sgemm(NN_BF16, B, d.C, d.K, P, 1, CLRows{act + off[4], cs}, ModeS{P}, StoreBF16{F, (size_t)FF, d.K}, st);
-    pack_bf16_kernel<<<grid_elems((size_t)O * FF), 256, 0, st>>>((size_t)O * FF, params + d.off_wh, whb);
-    dim3 hg((O + DG_T - 1) / DG_T, (B + DG_T - 1) / DG_T);
-    dense_bf16_gemm_kernel<<<hg, 128, 0, st>>>(B, O, FF, F, whb, params + d.off_bh, lam_out, O);
-}
-
 }  // namespace sch
 
 using namespace sch;
@@ -815,7 +441,7 @@ size_t nn_workspace_bytes(const nn_shape* s, int B) {
     // forward activations + two gradient buffers of one activation each + glam/gF + split-K partials
     const size_t generic = ((size_t)B * d.act_total * 3 + 2 * (size_t)d.C * d.K * B + (size_t)d.K * d.Ns * B +
                             partial_floats(d, B)) * sizeof(float);
-    return cf_supported(d) ? max(generic, cf_workspace_bytes(d, B)) : generic;
+    return max(generic, max(cf_supported(d) ? cf_workspace_bytes(d, B) : 0, cl_supported(d) ? cl_workspace_bytes(d, B) : 0));
 }
 
 static int nn_check(const nn_shape* s, int B, const void* params, const void* u, const void* y, void* ws,
@@ -833,10 +459,7 @@ int nn_forward(const nn_shape* s, int B, const float* params, const float* u_sta
     if (!lam_out || y_stride < 0) return SCH_ERR_ARG;
     const NNDims d = make_dims(s);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (cl_supported(d)) {
-        nn_forward_cl(d, B, params, u_start, y, y_stride, ws, lam_out, st);
-        return cudaGetLastError() == cudaSuccess ? SCH_OK : SCH_ERR_CUDA;
-    }
+    if (cl_supported(d)) return nn_forward_cl(d, B, params, u_start, y, y_stride, ws, lam_out, st);
     float* act = reinterpret_cast<float*>(ws);
     nn_forward_impl(d, B, params, u_start, y, y_stride, act, st);
     const int O = d.K * d.Ns;
