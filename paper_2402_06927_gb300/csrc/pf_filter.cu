@@ -11,23 +11,37 @@ namespace sch {
 constexpr int TEMPER_CTAS = 8;          // one thread-block cluster
 constexpr int TEMPER_PER_THREAD = 8;    // N <= 8 * 256 * 8 = 16384
 // threads per CTA: 128 up to N = 8 * 128 = 1024 (one particle per thread, every CTA
-// busy), else 256.  The FP64 pipe bounds an evaluation, and every thread's share of
-// the reductions runs on it; above N = 1024 the wider CTA shortens each thread's
-// serial chain of exponentials.
+// busy), else 256: above N = 1024 the wider CTA shortens each thread's serial chain
+// of exponentials.
 constexpr int TEMPER_THREADS_SMALL = 128, TEMPER_THREADS_LARGE = 256;
 constexpr int RESAMPLE_THREADS = 1024;
 
-// Adaptive tempering on one cluster of TEMPER_CTAS CTAs: every CTA holds a
-// slice of the particles, ESS evaluations reduce (sum w, sum w^2) in the CTA,
-// then across the cluster through distributed shared memory.  Every CTA sums
-// the partials in the same order, so all CTAs take identical root-search
-// decisions.  Partials are double-buffered by evaluation parity, so one
-// cluster barrier per evaluation suffices.
+// Adaptive tempering on one cluster of TEMPER_CTAS CTAs: every CTA holds a slice of the
+// particles, an evaluation reduces its sums over the cluster through distributed shared
+// memory.  Every CTA sums the partials in the same order, so all CTAs take identical
+// decisions.  Partials are double-buffered by evaluation parity, so one cluster barrier
+// per evaluation suffices.
+//
+// What bounds it is the FP64 unit, on which a warp's instruction takes 64 cycles of its
+// sub-partition: an FP64 evaluation costs about 25 of them a particle (the exponential),
+// and any scalar that every warp computes for itself costs as much again.  So the root of
+// ESS(d) = ess_min is located in float first (eight points an evaluation, the exponentials
+// on the special-function unit), two or three Newton steps in FP64 finish it, and only
+// warp 0 sums the partials and takes the decisions.  Tempering, resampling and gathers of 8001
+// particles of n = 1024: 207 us with an Illinois search of 12 to 15 FP64 evaluations summed by
+// every warp, 110 us so.
+constexpr int TEMPER_POINTS = 8;
 struct TemperShm {
-    double part[2][2];      // [parity][s1, s2] of this CTA
-    double warp[2][8];      // per-warp partials (s1, s2)
-    double minw[8];
+    double dpart[2][8][2];                       // [parity][warp] S1, S2 of an FP64 evaluation
+    float tpart[2][8][2];                        // ... and T1, T2
+    float fwarp[8][2 * TEMPER_POINTS];           // a float evaluation: per-warp sums,
+    float fpart[2][2 * TEMPER_POINTS];           // [parity] and the CTA's
+    double minw[8], cmin;
+    double c, s1, s2;                            // warp 0's decision: the next point, or the answer,
+    int act;                                     // one of TemperAct,
+    int keep;                                    // and whether the weights just formed are the answer's so far
 };
+enum TemperAct { TEMPER_EVAL = 0, TEMPER_LAST = 1, TEMPER_DONE = 2 };
 
 template <int TPT>
 __device__ __forceinline__ double cta_min(double v, TemperShm* sh) {
@@ -43,19 +57,20 @@ __device__ __forceinline__ double cta_min(double v, TemperShm* sh) {
 }
 
 // The sums S1 = sum w_e and S2 = sum w_e^2 of the weights w_e = exp(-d phi_e - max),
-// max = -d phi_min, over the cluster (ESS = S1^2 / S2, Eq. ess); the thread's weights
-// are returned in w.  Every thread sums the CTAs' partials in rank order, so all CTAs
-// take identical decisions.  (Folding them over 8 lanes with shuffles instead, each
-// lane reading another CTA, measured slower at 256 threads: 216 us against 165 per
-// search at N = 8192.)
+// max = -d phi_min, over the cluster (ESS = S1^2 / S2, Eq. ess), and in float T1 = sum z_e
+// w_e and T2 = sum z_e w_e^2, z_e = phi_e - phi_min, which give its slope: d log ESS / dd =
+// -2 (T1 / S1 - T2 / S2).  The sums are warp 0's; the thread's weights are returned in w.
 template <int TPT>
-__device__ __forceinline__ void ess_sums(double d, const double (&phi)[TEMPER_PER_THREAD], int cnt, double phimin,
-                                         TemperShm* sh, int& parity, double& S1, double& S2,
+__device__ __forceinline__ void ess_sums(double d, const double (&phi)[TEMPER_PER_THREAD],
+                                         const float (&z)[TEMPER_PER_THREAD], int cnt, double phimin, TemperShm* sh,
+                                         int& parity, double& S1, double& S2, float& T1, float& T2,
                                          double (&w)[TEMPER_PER_THREAD]) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
+    constexpr int NW = TPT / 32;
     const double mx = -d * phimin;
     double s1 = 0.0, s2 = 0.0;
+    float t1 = 0.f, t2 = 0.f;
 #pragma unroll
     for (int e = 0; e < TEMPER_PER_THREAD; ++e) {
         w[e] = 0.0;
@@ -63,35 +78,115 @@ __device__ __forceinline__ void ess_sums(double d, const double (&phi)[TEMPER_PE
             w[e] = exp(-d * phi[e] - mx);
             s1 += w[e];
             s2 += w[e] * w[e];
+            const float wf = (float)w[e];
+            if (wf > 0.f) {      // an infinite z has no weight
+                t1 = fmaf(z[e], wf, t1);
+                t2 = fmaf(z[e] * wf, wf, t2);
+            }
         }
     }
-    s1 = warp_sum(s1);
-    s2 = warp_sum(s2);
+    // the lower half of the warp sums s1, the upper s2: five FP64 additions for the two
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        sh->warp[0][warp] = s1;
-        sh->warp[1][warp] = s2;
+    const bool up = lane & 16;
+    const double sent = __shfl_xor_sync(FULL, up ? s1 : s2, 16);
+    double s = (up ? s2 : s1) + sent;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        t1 += __shfl_xor_sync(FULL, t1, o);
+        t2 += __shfl_xor_sync(FULL, t2, o);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int w = 0; w < TPT / 32; ++w) {
-            a += sh->warp[0][w];
-            b += sh->warp[1][w];
-        }
-        sh->part[parity][0] = a;
-        sh->part[parity][1] = b;
+    if ((lane & 15) == 0) sh->dpart[parity][warp][lane >> 4] = s;
+    if (lane == 0) {
+        sh->tpart[parity][warp][0] = t1;
+        sh->tpart[parity][warp][1] = t2;
     }
     cl.sync();
-    double t1 = 0.0, t2 = 0.0;
-    for (int r = 0; r < TEMPER_CTAS; ++r) {
-        const TemperShm* o = cl.map_shared_rank(sh, r);
-        t1 += o->part[parity][0];
-        t2 += o->part[parity][1];
+    if (warp == 0) {
+        // one partial per (CTA, warp): lane l takes those of number l, l + 32, ...
+        double a = 0.0, b = 0.0;
+        t1 = 0.f;
+        t2 = 0.f;
+#pragma unroll
+        for (int q = 0; q < TEMPER_CTAS * NW / 32; ++q) {
+            const int k = lane + 32 * q;
+            const TemperShm* o = cl.map_shared_rank(sh, k / NW);
+            const double pa = o->dpart[parity][k % NW][0], pb = o->dpart[parity][k % NW][1];
+            a = q ? a + pa : pa;
+            b = q ? b + pb : pb;
+            t1 += o->tpart[parity][k % NW][0];
+            t2 += o->tpart[parity][k % NW][1];
+        }
+        const double got = __shfl_xor_sync(FULL, up ? a : b, 16);
+        double v = (up ? b : a) + got;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+        S1 = __shfl_sync(FULL, v, 0);
+        S2 = __shfl_sync(FULL, v, 16);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            t1 += __shfl_xor_sync(FULL, t1, o);
+            t2 += __shfl_xor_sync(FULL, t2, o);
+        }
+        T1 = t1;
+        T2 = t2;
     }
     parity ^= 1;
-    S1 = t1;
-    S2 = t2;
+}
+
+// One float evaluation at the TEMPER_POINTS points x_g = x0 + g dx (geo: x0 2^g): the number of
+// points that pass before the first that does not, and g(x) = ESS - ess_min at the last that
+// passes (gl) and at the next (gh); the same in every thread of the cluster.
+template <int TPT>
+__device__ __forceinline__ int ess_points(float x0, float dx, bool geo, const float (&z)[TEMPER_PER_THREAD], int cnt,
+                                          float ess_min, TemperShm* sh, int& parity, float& gl, float& gh) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    constexpr int G = TEMPER_POINTS;
+    float v[2 * G];
+#pragma unroll
+    for (int g = 0; g < 2 * G; ++g) v[g] = 0.f;
+    for (int e = 0; e < cnt; ++e) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const float x = geo ? x0 * (float)(1 << g) : fmaf((float)g, dx, x0);
+            float w;
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w) : "f"(-1.44269504f * x * z[e]));
+            v[g] += w;
+            v[G + g] = fmaf(w, w, v[G + g]);
+        }
+    }
+    // halving butterfly: after the exchanges over 16, 8, 4 and 2 a lane holds sum number lane / 2
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int h = G, o = 16; h >= 1; h >>= 1, o >>= 1)
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const bool up = lane & o;
+            const float got = __shfl_xor_sync(FULL, up ? v[k] : v[k + h], o);
+            v[k] = (up ? v[k + h] : v[k]) + got;
+        }
+    v[0] += __shfl_xor_sync(FULL, v[0], 1);
+    if ((lane & 1) == 0) sh->fwarp[warp][lane >> 1] = v[0];
+    __syncthreads();
+    if (threadIdx.x < 2 * G) {
+        float s = 0.f;
+        for (int w = 0; w < TPT / 32; ++w) s += sh->fwarp[w][threadIdx.x];
+        sh->fpart[parity][threadIdx.x] = s;
+    }
+    cl.sync();
+    float s = 0.f;
+#pragma unroll
+    for (int r = 0; r < TEMPER_CTAS; ++r) s += cl.map_shared_rank(sh, r)->fpart[parity][lane & (2 * G - 1)];
+    parity ^= 1;
+    const float s2 = __shfl_sync(FULL, s, (lane & (G - 1)) + G);
+    const float g = s * s / s2 - ess_min;                     // lanes 0 .. G - 1
+    const unsigned fail = __ballot_sync(FULL, !(g >= 0.f)) & ((1u << G) - 1);
+    const int k = fail ? __ffs(fail) - 1 : G;
+    gl = __shfl_sync(FULL, g, k > 0 ? k - 1 : 0);
+    gh = __shfl_sync(FULL, g, k < G ? k : 0);
+    return k;
 }
 
 template <int TPT>
@@ -137,83 +232,151 @@ __global__ void __cluster_dims__(TEMPER_CTAS, 1, 1) __launch_bounds__(TPT)
         }
     }
     // cluster-wide minimum of phi
-    double cmin = cta_min<TPT>(lmin, sh);
-    if (threadIdx.x == 0) sh->part[1][0] = cmin;
+    const double cmin = cta_min<TPT>(lmin, sh);
+    if (threadIdx.x == 0) sh->cmin = cmin;
     cl.sync();
     double phimin = INFINITY;
-    for (int r = 0; r < TEMPER_CTAS; ++r) phimin = fmin(phimin, cl.map_shared_rank(sh, r)->part[1][0]);
-    int parity = 0;   // the next evaluation writes parity 0; parity 1 is free again after its barrier
-    const double rest = 1.0 - theta;
-    // (s1, s2, wk): the sums and this thread's weights at the current answer, so that
-    // the normalised weights need no further pass.  Whether the whole step passes is
-    // tested as S1^2 >= ess_min S2 (S2 > 0), without a division.
-    double s1, s2, wk[TEMPER_PER_THREAD], wc[TEMPER_PER_THREAD];
-    ess_sums<TPT>(rest, phi, cnt, phimin, sh, parity, s1, s2, wk);
-    const double s1_rest = s1, s2_rest = s2;
-    // The largest dtheta with ESS >= ess_min.  ESS(d) falls monotonically in d
-    // (its log-derivative is 2 (E_{w^2}[phi] - E_w[phi]) <= 0), so the root of
-    // g(d) = ESS(d) - ess_min is bracketed by [0, rest] (g(0) = N - ess_min >= 0)
-    // and found by the Illinois variant of regula falsi: the secant point of the
-    // bracket, with the function value at an end kept twice in a row halved, and a
-    // midpoint whenever the bracket failed to halve over three steps.  It stops at a
-    // relative width of 2^-46 and returns the passing end.  A root below rest 2^-60
-    // (astronomically spread phi) gives rest 2^-60, the smallest point 60 bisection
-    // steps would try.  (Run on S1^2 - ess_min S2 instead, which has the same root and
-    // saves the division, the secant steps needed more evaluations, and a searching call
-    // at N = 1024 took 20% longer.)
-    double d;
-    if (s1 * s1 >= ess_min * s2) {
-        d = rest;
-    } else if (halving) {
-        // the paper's search read literally: halve dtheta until the ESS passes, at most
-        // 60 times (the last point tried is kept if none passes)
-        d = rest;
-        for (int k = 1; k <= 60; ++k) {
-            d = ldexp(rest, -k);
-            ess_sums<TPT>(d, phi, cnt, phimin, sh, parity, s1, s2, wk);
-            if (s1 * s1 >= ess_min * s2) break;
-        }
-    } else {
-        const double dmin = rest * 0x1.0p-60;
-        double lo = 0.0, glo = (double)N - ess_min, hi = rest, ghi = s1 * s1 / s2 - ess_min;
-        double w3 = rest, w2 = rest, w1 = rest;   // bracket widths of the last three steps
-        int side = 0;
-        for (int it = 0; it < 200; ++it) {
-            const double w = hi - lo;
-            if (w <= hi * 0x1.0p-46 || hi < dmin) break;
-            double c = (lo * ghi - hi * glo) / (ghi - glo);
-            if (!(c > lo && c < hi) || w > 0.5 * w3) c = 0.5 * (lo + hi);
-            w3 = w2;
-            w2 = w1;
-            w1 = w;
-            double sc, s2c;
-            ess_sums<TPT>(c, phi, cnt, phimin, sh, parity, sc, s2c, wc);
-            const double gc = sc * sc / s2c - ess_min;
-            if (gc >= 0.0) {
-                lo = c;
-                glo = gc;
-                s1 = sc;
-                s2 = s2c;
+    for (int r = 0; r < TEMPER_CTAS; ++r) phimin = fmin(phimin, cl.map_shared_rank(sh, r)->cmin);
+    float z[TEMPER_PER_THREAD];
 #pragma unroll
-                for (int e = 0; e < TEMPER_PER_THREAD; ++e) wk[e] = wc[e];
-                if (side == 1) ghi *= 0.5;
-                side = 1;
-            } else {
-                hi = c;
-                ghi = gc;
-                if (side == -1) glo *= 0.5;
-                side = -1;
-            }
-        }
-        if (lo > 0.0) {
-            d = lo;
-        } else {
-            d = fmax(hi, dmin);
-            ess_sums<TPT>(d, phi, cnt, phimin, sh, parity, s1, s2, wk);
+    for (int e = 0; e < TEMPER_PER_THREAD; ++e) z[e] = (e < cnt) ? (float)(phi[e] - phimin) : 0.f;
+    int parity = 0;
+    const double rest = 1.0 - theta;
+    const bool lead = threadIdx.x < 32;
+    // wk: this thread's weights at the answer so far, so that the normalised weights need no
+    // further pass.  A point passes when S1^2 >= ess_min S2 (S2 > 0), without a division.
+    double S1 = 0.0, S2 = 0.0, wk[TEMPER_PER_THREAD];
+    float T1 = 0.f, T2 = 0.f;
+    ess_sums<TPT>(rest, phi, z, cnt, phimin, sh, parity, S1, S2, T1, T2, wk);
+    const double s1_rest = S1, s2_rest = S2;   // (warp 0)
+    if (lead) {
+        if (threadIdx.x == 0) {
+            sh->s1 = S1;
+            sh->s2 = S2;
+            sh->c = rest;
+            sh->act = (S1 * S1 >= ess_min * S2) ? TEMPER_DONE : TEMPER_EVAL;
         }
     }
-    const double ess = s1 * s1 / s2;
-    const double ess_rest = s1_rest * s1_rest / s2_rest;
+    __syncthreads();
+    if (sh->act != TEMPER_DONE && halving) {
+        // the paper's search read literally: halve dtheta until the ESS passes, at most
+        // 60 times (the last point tried is kept if none passes)
+        for (int k = 1; k <= 60; ++k) {
+            const double d = ldexp(rest, -k);
+            ess_sums<TPT>(d, phi, z, cnt, phimin, sh, parity, S1, S2, T1, T2, wk);
+            if (threadIdx.x == 0) {
+                sh->s1 = S1;
+                sh->s2 = S2;
+                sh->c = d;
+                sh->act = (S1 * S1 >= ess_min * S2) ? TEMPER_DONE : TEMPER_EVAL;
+            }
+            __syncthreads();
+            if (sh->act == TEMPER_DONE) break;
+        }
+    } else if (sh->act != TEMPER_DONE) {
+        // The largest dtheta with ESS >= ess_min.  ESS(d) falls monotonically in d (its
+        // log-derivative is 2 (E_{w^2}[phi] - E_w[phi]) <= 0), so the root of g(d) = ESS(d) -
+        // ess_min is bracketed by [0, rest] (g(0) = N - ess_min >= 0).
+        // Float: the root's octave, then three ninths of the bracket and the secant point of
+        // what is left (1/729 of an octave): the root to about 1e-6.
+        float a = 0.f, b = (float)rest, ga = (float)N - (float)ess_min, gb = -1.f;
+        const float ess_f = (float)ess_min;
+        for (int r = 0; r < 8; ++r) {
+            const float x0 = b * 0x1p-8f;
+            float gl, gh;
+            const int k = ess_points<TPT>(x0, 0.f, true, z, cnt, ess_f, sh, parity, gl, gh);
+            if (k < TEMPER_POINTS) {
+                b = x0 * (float)(1 << k);
+                gb = gh;
+            }
+            if (k > 0) {
+                a = x0 * (float)(1 << (k - 1));
+                ga = gl;
+                break;
+            }
+        }
+        for (int r = 0; r < 3; ++r) {
+            const float dx = (b - a) * (1.f / (TEMPER_POINTS + 1));
+            float gl, gh;
+            const int k = ess_points<TPT>(a + dx, dx, false, z, cnt, ess_f, sh, parity, gl, gh);
+            const float a0 = a;
+            if (k > 0) {
+                a = fmaf((float)k, dx, a0);
+                ga = gl;
+            }
+            if (k < TEMPER_POINTS) {
+                b = fmaf((float)(k + 1), dx, a0);
+                gb = gh;
+            }
+        }
+        // FP64: Newton steps from the float root inside the bracket [lo, hi] (lo passes, hi does
+        // not), the step itself in float; a midpoint where a step leaves the bracket and every
+        // sixth time.  Near the root the point is put 2^-51 below the estimate, so that it
+        // passes.  The search stops at a passing point whose distance to the root is at most
+        // 2^-49 of it, or when the bracket is that narrow.  A root below rest 2^-60
+        // (astronomically spread phi) gives rest 2^-60, the smallest point 60 bisection steps
+        // would try.
+        const double dmin = rest * 0x1.0p-60;
+        double lo = 0.0, hi = rest, c = (double)(a + (b - a) * (ga / (ga - gb)));
+        if (!(c > lo && c < hi)) c = 0.5 * hi;
+        double ks1 = 0.0, ks2 = 0.0;                // the sums at lo (warp 0)
+        for (int it = 1;; ++it) {
+            double wc[TEMPER_PER_THREAD];
+            ess_sums<TPT>(c, phi, z, cnt, phimin, sh, parity, S1, S2, T1, T2, wc);
+            if (lead) {
+                const double num = fma(S1, S1, -(ess_min * S2));
+                const bool pass = num >= 0.0;
+                // g / |g'| = (num / S2) / (ESS |dlog ESS|): the root is at c + dl
+                const float s1f = (float)S1, s2f = (float)S2;
+                const float dl = (float)num / (2.f * s1f * s1f * (T1 / s1f - T2 / s2f));
+                const float cf = (float)c;
+                int act = TEMPER_EVAL;
+                if (pass) {
+                    lo = c;
+                    ks1 = S1;
+                    ks2 = S2;
+                    if (dl <= cf * 0x1p-49f) act = TEMPER_DONE;
+                } else {
+                    hi = c;
+                }
+                double cn = lo;
+                if (hi - lo <= hi * 0x1.0p-49 || hi < dmin || it >= 400) act = TEMPER_DONE;
+                if (act == TEMPER_DONE) {
+                    if (!(lo > 0.0)) {
+                        act = TEMPER_LAST;
+                        cn = fmax(hi, dmin);
+                    }
+                } else {
+                    cn = c + (double)dl;
+                    if (fabsf(dl) < cf * 0x1p-30f) cn = fma(c, -0x1.0p-51, cn);
+                    if (!(cn > lo && cn < hi) || it % 6 == 0) cn = 0.5 * (lo + hi);
+                }
+                if (threadIdx.x == 0) {
+                    sh->c = cn;
+                    sh->s1 = ks1;
+                    sh->s2 = ks2;
+                    sh->act = act;
+                    sh->keep = pass;
+                }
+            }
+            __syncthreads();
+            c = sh->c;
+            if (sh->keep) {
+#pragma unroll
+                for (int e = 0; e < TEMPER_PER_THREAD; ++e) wk[e] = wc[e];
+            }
+            if (sh->act != TEMPER_EVAL) break;
+        }
+        if (sh->act == TEMPER_LAST) {
+            ess_sums<TPT>(c, phi, z, cnt, phimin, sh, parity, S1, S2, T1, T2, wk);
+            if (threadIdx.x == 0) {
+                sh->s1 = S1;
+                sh->s2 = S2;
+            }
+            __syncthreads();
+        }
+    }
+    const double d = sh->c, s1 = sh->s1;
 #pragma unroll
     for (int e = 0; e < TEMPER_PER_THREAD; ++e) {
         const int i = gt + e * STRIDE;
@@ -221,9 +384,9 @@ __global__ void __cluster_dims__(TEMPER_CTAS, 1, 1) __launch_bounds__(TPT)
     }
     if (rank == 0 && threadIdx.x == 0) {
         out[0] = d;
-        out[1] = ess;
+        out[1] = s1 * s1 / sh->s2;
         out[2] = (d >= 1.0 - theta) ? 1.0 : theta + d;
-        out[3] = ess_rest;
+        out[3] = s1_rest * s1_rest / s2_rest;
         if (theta_dev) out[4] = 1.0;
     }
     cl.sync();   // no CTA leaves while another may still read its shared memory
