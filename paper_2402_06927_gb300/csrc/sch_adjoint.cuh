@@ -86,43 +86,6 @@ __device__ __forceinline__ void var_solve(const R (&a)[C], const R (&b)[C], cons
     for (int i = 1; i < C - 1; ++i) x[i] = de[i] - al[i] * F - ga[i] * E;
 }
 
-// neighbours of two chunk fields at once (E/F and hE/hF as exchange slots)
-template <typename R, int C, int TP>
-__device__ __forceinline__ void chunk_halo2(const R (&v)[C], R& vp, R& vn, const R (&w)[C], R& wp, R& wn,
-                                           Shm<R, TP>* sh) {
-    const int t = threadIdx.x;
-    sh->E[t] = v[C - 1];
-    sh->F[t] = v[0];
-    sh->hE[t] = w[C - 1];
-    sh->hF[t] = w[0];
-    __syncthreads();
-    vp = sh->E[(t - 1) & (TP - 1)];
-    vn = sh->F[(t + 1) & (TP - 1)];
-    wp = sh->hE[(t - 1) & (TP - 1)];
-    wn = sh->hF[(t + 1) & (TP - 1)];
-    __syncthreads();
-}
-
-// max over the CTA (all threads receive it); one barrier pair
-template <typename R, int TP>
-__device__ __forceinline__ void block_max2_all(Shm<R, TP>* sh, R& a, R& b) {
-    a = warp_max(a);
-    b = warp_max(b);
-    const int t = threadIdx.x;
-    if ((t & 31) == 0) {
-        sh->wred[0][t >> 5] = a;
-        sh->wred[1][t >> 5] = b;
-    }
-    __syncthreads();
-    a = sh->wred[0][0];
-    b = sh->wred[1][0];
-    for (int w = 1; w < TP / 32; ++w) {
-        a = fmax(a, sh->wred[0][w]);
-        b = fmax(b, sh->wred[1][w]);
-    }
-    __syncthreads();
-}
-
 // --------------------------------------------------------------------------
 // Adjoint of one converged step.  In: the step's states (m0, u0) -> (m1, u1)
 // with chunk-end neighbours, dU/4 at nodes i0-1 .. i0+C, and g = dJ/dm1 (with
@@ -181,14 +144,10 @@ __device__ __forceinline__ void adjoint_step(const ModelArgs<R>& A, Shm<R, TP>* 
             const R Sl = (i == 0) ? Sp : S[i - 1];
             BT[i] = R(0.5) * (Sl * xl - S[i] * xr);
         }
-        // corr = (dt/2) M H^{-1} B^T psi
-        R q[C], qp, qn, r[C];
-        const_solve<R, C, TP>(A.hel, A.rhel, BT, q, qp, qn, sh);
-        mass_apply<R, C>(A.h6, q, qp, qn, r);
+        // the warp's maxima of the change and of psi, read after the Helmholtz solve's barriers
         R dmax = R(0), pmax = R(0);
 #pragma unroll
         for (int i = 0; i < C; ++i) {
-            corr[i] = R(0.5) * A.dt * r[i];
             R dd = rabs(pn[i] - psi[i]);
             if (!(dd == dd)) dd = R(INFINITY);
             dmax = fmax(dmax, dd);
@@ -197,7 +156,24 @@ __device__ __forceinline__ void adjoint_step(const ModelArgs<R>& A, Shm<R, TP>* 
         }
         psip = pnp;
         psin = pnn;
-        block_max2_all<R, TP>(sh, dmax, pmax);
+        dmax = warp_max_abs(dmax);
+        pmax = warp_max_abs(pmax);
+        if ((threadIdx.x & 31) == 0) {
+            sh->wred[0][threadIdx.x >> 5] = dmax;
+            sh->wred[1][threadIdx.x >> 5] = pmax;
+        }
+        // corr = (dt/2) M H^{-1} B^T psi
+        R q[C], qp, qn, r[C];
+        const_solve<R, C, TP>(A.hel, A.rhel, BT, q, qp, qn, sh);
+        mass_apply<R, C>(A.h6, q, qp, qn, r);
+#pragma unroll
+        for (int i = 0; i < C; ++i) corr[i] = R(0.5) * A.dt * r[i];
+        dmax = sh->wred[0][0];
+        pmax = sh->wred[1][0];
+        for (int k = 1; k < TP / 32; ++k) {
+            dmax = fmax(dmax, sh->wred[0][k]);
+            pmax = fmax(pmax, sh->wred[1][k]);
+        }
         iters++;
         if (!(dmax < R(INFINITY)) || !(pmax < R(INFINITY))) {
             flags |= SCH_DEV_NONFINITE;
@@ -443,35 +419,72 @@ __device__ __forceinline__ bool adjoint_step_refined(const ModelArgs<double>& A,
     return true;
 }
 
-// sum over the CTA of sin(j theta_i) x_i and cos(j theta_i) x_i, j = 1 .. K/2:
-// each warp reduces with shuffles and lane 0 writes red[warp * K + 2(j-1) (+1)];
-// the caller sums over warps after a barrier.  (s1, c1): angle of node i0.
+// exact float -> double on the integer pipe (a conversion instruction runs on the narrow FP64
+// unit); subnormals, infinities and NaN take the instruction
+__device__ __forceinline__ double f2d_exact(float x) {
+    const unsigned b = __float_as_uint(x), ab = b & 0x7fffffffu;
+    if (ab - 0x00800000u >= 0x7f000000u) return (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | ((ab >> 3) + (896u << 20))), (int)(b << 29));
+}
+
+// eight warp sums at once, number lane >> 2 left in v[0] of every lane (9 additions)
+__device__ __forceinline__ void warp_sums8(double (&v)[8]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1)
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const bool up = lane & o;
+            const double keep = up ? v[k + h] : v[k], send = up ? v[k] : v[k + h];
+            v[k] = keep + __shfl_xor_sync(FULL, send, o);
+        }
+    v[0] += __shfl_xor_sync(FULL, v[0], 2);
+    v[0] += __shfl_xor_sync(FULL, v[0], 1);
+}
+
+// sum over the CTA of sin(j theta_i) x_i and cos(j theta_i) x_i, j = 1 .. K/2, of a float
+// field: each warp adds its lanes' partial sums in double and writes red[warp * K + 2(j-1)
+// (+1)]; the caller sums over warps after a barrier.  (s1, c1): angle of node i0.
+// A warp's double addition holds the narrow FP64 unit for 64 cycles, so four harmonics' eight
+// sums cross the warp in one halving butterfly: 9 additions for what took 40 as eight
+// butterflies of their own (with two conversions a harmonic).  With the stop test's maxima read
+// after the Helmholtz solve's barriers (four barriers an iteration instead of six), the
+// chunk-end neighbours read from the kept rows and vector accesses in warp 0, 301 gradients
+// at n = 1024, 17 steps, checkpoints every 7: 453 -> 361 us; 512 nudged particles at n = 1024:
+// 18.7 -> 16.4 ms.
 template <typename R, int C>
 __device__ __forceinline__ void mode_sums_warp(const ModelArgs<R>& A, R s1, R c1, const R (&x)[C], double* red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const R twoc = R(2) * c1;
     R sj = s1, cj = c1, sjm = R(0), cjm = R(1);
-    for (int j = 0; j < A.K2; ++j) {
-        const R rc = A.rot_c[j], rs = A.rot_s[j];
-        R sn = sj, cs = cj, as = R(0), ac = R(0);
+    for (int j0 = 0; j0 < A.K2; j0 += 4) {
+        double v[8];
 #pragma unroll
-        for (int q = 0; q < C; ++q) {
-            as += sn * x[q];
-            ac += cs * x[q];
-            const R s2 = sn * rc + cs * rs;
-            cs = cs * rc - sn * rs;
-            sn = s2;
+        for (int h = 0; h < 4; ++h) {
+            R as = R(0), ac = R(0);
+            if (j0 + h < A.K2) {
+                const R rc = A.rot_c[j0 + h], rs = A.rot_s[j0 + h];
+                R sn = sj, cs = cj;
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    as += sn * x[q];
+                    ac += cs * x[q];
+                    const R s2 = sn * rc + cs * rs;
+                    cs = cs * rc - sn * rs;
+                    sn = s2;
+                }
+                const R sn2 = twoc * sj - sjm, cn2 = twoc * cj - cjm;
+                sjm = sj;
+                cjm = cj;
+                sj = sn2;
+                cj = cn2;
+            }
+            v[2 * h] = f2d_exact(as);
+            v[2 * h + 1] = f2d_exact(ac);
         }
-        const double das = warp_sum((double)as), dac = warp_sum((double)ac);
-        if (lane == 0) {
-            red[warp * A.K + 2 * j] = das;
-            red[warp * A.K + 2 * j + 1] = dac;
-        }
-        const R sn2 = twoc * sj - sjm, cn2 = twoc * cj - cjm;
-        sjm = sj;
-        cjm = cj;
-        sj = sn2;
-        cj = cn2;
+        warp_sums8(v);
+        const int o = 2 * j0 + (lane >> 2);
+        if ((lane & 3) == 0 && o < 2 * A.K2) red[warp * A.K + o] = v[0];
     }
 }
 
@@ -567,22 +580,27 @@ __device__ __forceinline__ void matern_adjoint_cells(const ModelArgs<R>& A, Shm<
     for (int i = 0; i < C; ++i) gw[i] = b * (x[i] + ((i == C - 1) ? xn : x[i + 1]));
 }
 
-// The states (m, u) around step s, kept as four rows of n at sl, with chunk-end neighbours, and
-// the step's noise
+// The states (m, u) around step s, kept as four rows of n = C TP (a power of two) values at
+// sl, with chunk-end neighbours, and the step's noise
 template <typename R, int C, int TP, int NZ>
 __device__ __forceinline__ void adjoint_load(const ModelArgs<R>& A, Shm<R, TP>* sh, const R* sl, R* noise,
                                              const R* dW, const R* lam, int s, R s0, R c0, StepState<R, C>& st,
                                              R (&nq)[C + 2]) {
+    // the rows were written by this CTA, the last of a recomputed segment with no barrier since
+    __syncthreads();
     load_field<R, C>(sl, st.m0);
     load_field<R, C>(sl + A.n, st.u0);
     load_field<R, C>(sl + 2 * A.n, st.m1);
     load_field<R, C>(sl + 3 * A.n, st.u1);
-    // the exchange below writes the slots hE, hF, which other warps may still be
-    // reading after the last barrier of a recomputed step or of the previous step's
-    // Matern solves
-    __syncthreads();
-    chunk_halo2<R, C, TP>(st.m0, st.m0p, st.m0n, st.u0, st.u0p, st.u0n, sh);
-    chunk_halo2<R, C, TP>(st.m1, st.m1p, st.m1n, st.u1, st.u1p, st.u1n, sh);
+    const int ip = ((int)threadIdx.x * C + A.n - 1) & (A.n - 1), in = ((int)threadIdx.x * C + C) & (A.n - 1);
+    st.m0p = sl[ip];
+    st.u0p = sl[A.n + ip];
+    st.m1p = sl[2 * A.n + ip];
+    st.u1p = sl[3 * A.n + ip];
+    st.m0n = sl[in];
+    st.u0n = sl[A.n + in];
+    st.m1n = sl[2 * A.n + in];
+    st.u1n = sl[3 * A.n + in];
     if constexpr (NZ == SCH_NOISE_MATERN) {
         matern_stage_step<R, C>(A, noise, dW, lam, s);
         matern_nodes<R, C, TP>(A, sh, noise, nq);

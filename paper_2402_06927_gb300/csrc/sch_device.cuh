@@ -191,4 +191,46 @@ __device__ __forceinline__ R warp_sum(R v) {
     return v;
 }
 
+// warp_max of values >= 0 (no NaN): floats in one instruction, as their bit patterns
+__device__ __forceinline__ float warp_max_abs(float v) {
+    return __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(v) & 0x7fffffffu));
+}
+__device__ __forceinline__ double warp_max_abs(double v) { return warp_max(v); }
+
+// a lane's RR consecutive values of a shared array (16-byte aligned), floats as vectors: scalar
+// accesses at a stride of RR words would conflict RR ways
+template <int RR, typename R>
+__device__ __forceinline__ void rows_load(const R* p, R (&v)[RR]) {
+    if constexpr (sizeof(R) == 4 && RR % 4 == 0) {
+#pragma unroll
+        for (int r = 0; r < RR; r += 4) {
+            const float4 a = *reinterpret_cast<const float4*>(p + r);
+            v[r] = a.x;
+            v[r + 1] = a.y;
+            v[r + 2] = a.z;
+            v[r + 3] = a.w;
+        }
+    } else if constexpr (sizeof(R) == 4 && RR == 2) {
+        const float2 a = *reinterpret_cast<const float2*>(p);
+        v[0] = a.x;
+        v[1] = a.y;
+    } else {
+#pragma unroll
+        for (int r = 0; r < RR; ++r) v[r] = p[r];
+    }
+}
+template <int RR, typename R>
+__device__ __forceinline__ void rows_store(R* p, const R (&v)[RR]) {
+    if constexpr (sizeof(R) == 4 && RR % 4 == 0) {
+#pragma unroll
+        for (int r = 0; r < RR; r += 4)
+            *reinterpret_cast<float4*>(p + r) = make_float4(v[r], v[r + 1], v[r + 2], v[r + 3]);
+    } else if constexpr (sizeof(R) == 4 && RR == 2) {
+        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    } else {
+#pragma unroll
+        for (int r = 0; r < RR; ++r) p[r] = v[r];
+    }
+}
+
 }  // namespace sch

@@ -38,7 +38,7 @@ namespace sch {
 // shared memory of one particle CTA
 // --------------------------------------------------------------------------
 template <typename R, int TP>
-struct Shm {
+struct __align__(16) Shm {
     static constexpr int RR = TP / 32 > 1 ? TP / 32 : 1;
     R pa[TP], pc[TP], pd[TP], ae[TP], ge[TP], de[TP];   // reduced rows of the Picard matrix
     R hpd[TP], hde[TP];                                  // reduced rows of a constant matrix
@@ -251,17 +251,11 @@ __device__ __forceinline__ void warp_solve_const(const CTab<R>& T, const RTab<R>
     constexpr int RR = TP / 32;
     const int t0 = (threadIdx.x & 31) * RR;
     R p[RR], d[RR], e[RR], f[RR];
-#pragma unroll
-    for (int r = 0; r < RR; ++r) {
-        p[r] = pd[t0 + r];
-        d[r] = de[t0 + r];
-    }
+    rows_load<RR>(pd + t0, p);
+    rows_load<RR>(de + t0, d);
     lane_solve_const<R, TP>(T, Q, p, d, e, f);
-#pragma unroll
-    for (int r = 0; r < RR; ++r) {
-        E[t0 + r] = e[r];
-        F[t0 + r] = f[r];
-    }
+    rows_store<RR>(E + t0, e);
+    rows_store<RR>(F + t0, f);
     __syncwarp();
 }
 
@@ -680,8 +674,8 @@ __device__ __forceinline__ void sch_step_ea(const ModelArgs<R>& A, Shm<R, TP>* s
                 constexpr int NW = TP / 32;
                 R dm = (t < NW) ? sh->wred[0][t] : R(0);
                 R mm = (t < NW) ? sh->wred[1][t] : R(0);
-                dm = warp_max(dm);
-                mm = warp_max(mm);
+                dm = warp_max_abs(dm);
+                mm = warp_max_abs(mm);
                 if (!(dm < R(INFINITY)) || !(mm < R(INFINITY))) fl = FLAG_STOP | FLAG_NONFINITE;
                 else if (ea_converged(dm, dm_prev, A.tol * fmax(R(1), mm))) fl = FLAG_STOP | FLAG_CONVERGED;
                 else if (it > A.max_iter) fl = FLAG_STOP | FLAG_NOCONV;
@@ -689,14 +683,10 @@ __device__ __forceinline__ void sch_step_ea(const ModelArgs<R>& A, Shm<R, TP>* s
             }
             if (!(fl & FLAG_STOP)) {
                 R pdr[RR], der[RR], hpr[RR], hdr[RR], Er[RR], Fr[RR];
-#pragma unroll
-                for (int r = 0; r < RR; ++r) {
-                    const int q = t * RR + r;
-                    pdr[r] = sh->pd[q];
-                    der[r] = sh->de[q];
-                    hpr[r] = sh->hpd[q];
-                    hdr[r] = sh->hde[q];
-                }
+                rows_load<RR>(sh->pd + t * RR, pdr);
+                rows_load<RR>(sh->de + t * RR, der);
+                rows_load<RR>(sh->hpd + t * RR, hpr);
+                rows_load<RR>(sh->hde + t * RR, hdr);
                 lane_solve_const<R, TP>(A.pic, A.rpic, pdr, der, Er, Fr);
                 // Helmholtz rows from the Picard interface values
                 const R Ep = __shfl_sync(FULL, Er[RR - 1], (t + 31) & 31);
@@ -710,14 +700,10 @@ __device__ __forceinline__ void sch_step_ea(const ModelArgs<R>& A, Shm<R, TP>* s
                 }
                 R hEr[RR], hFr[RR];
                 lane_solve_const<R, TP>(A.hel, A.rhel, hpr, hdr, hEr, hFr);
-#pragma unroll
-                for (int r = 0; r < RR; ++r) {
-                    const int q = t * RR + r;
-                    sh->E[q] = Er[r];
-                    sh->F[q] = Fr[r];
-                    sh->hE[q] = hEr[r];
-                    sh->hF[q] = hFr[r];
-                }
+                rows_store<RR>(sh->E + t * RR, Er);
+                rows_store<RR>(sh->F + t * RR, Fr);
+                rows_store<RR>(sh->hE + t * RR, hEr);
+                rows_store<RR>(sh->hF + t * RR, hFr);
             }
             if (t == 0) sh->flag = fl;
         }
@@ -758,8 +744,8 @@ __device__ __forceinline__ void sch_step_ea(const ModelArgs<R>& A, Shm<R, TP>* s
             mi[i] = mnew[i];
             ui[i] = un;
         }
-        dmax = warp_max(dmax);
-        mmax = warp_max(mmax);
+        dmax = warp_max_abs(dmax);
+        mmax = warp_max_abs(mmax);
         if ((t & 31) == 0) {
             sh->wred[0][t >> 5] = dmax;
             sh->wred[1][t >> 5] = mmax;
