@@ -20,6 +20,7 @@ struct sch_ctx {
     GArgs ga;
     ModelArgs<float> af;
     ModelArgs<double> ad;
+    ModelArgs<double> ad2;   // the tables of two-node chunks (sch_pairs_f64.cu): FP64, n <= 256
     void* jws;        // caller-owned jitter workspace (sch_set_jitter_workspace), or null
     size_t jws_bytes;
 };
@@ -591,6 +592,7 @@ int sch_create(const sch_params* params, sch_ctx** ctx) {
     c->Q = matern ? p.n : p.K;
     fill_args(p, C, c->af);
     fill_args(p, C, c->ad);
+    if (p.dtype == SCH_F64 && p.n <= 256) fill_args(p, 2, c->ad2);
     if (warp_ok) {
         // one warp per particle: 32 lanes x 2P sub-chunks of wcs nodes, a reduced system of 64 P rows
         const int P = warp_streams(p.n);
@@ -668,6 +670,22 @@ int sch_draw_increments(sch_ctx* ctx, int N, int nsteps, uint64_t seed, uint64_t
     return launch_draw<double>(N, nsteps, ctx->Q, sq, seed, tag, ctr, particle0, 0, (double*)dW, S(stream));
 }
 
+namespace {
+
+// Whether an FP64 launch of N particles runs on two-node chunks (sch_pairs_f64.cu): while an SM
+// holds at most three particles of 128 nodes or one of 256, so that their warps on two-node
+// chunks (nearly) all have an FP64 unit of their own.  Five steps, four-node against two-node
+// chunks, us (152 SMs): n = 128, N = 304 172 / 132, 456 173 / 155, 608 181 / 182; n = 256, N =
+// 152 172 / 138, 228 182 / 193; n = 512, N = 16 196 / 217 (the reduced solve of 256 rows
+// takes back more than the FP64 unit gives).
+bool use_pairs(const sch_ctx* ctx, int N, int nsteps, int bufs) {
+    if (ctx->p.dtype != SCH_F64 || ctx->ad.solver != SCH_SOLVER_LI || ctx->p.n > 256) return false;
+    if (N > (ctx->p.n == 128 ? 3 : 1) * device_sms()) return false;
+    return ctx->matern || pairs_smem(ctx->p.n, nsteps, ctx->Q, bufs) <= 200 * 1024;
+}
+
+}  // namespace
+
 int sch_ensemble_step(sch_ctx* ctx, int N, int nsteps, const void* m, void* m_out, void* u_out,
                       const void* dW, const void* lambda, const void* y, double* nll, double* logG,
                       int32_t* iters, int32_t* status, void* stream) {
@@ -696,6 +714,7 @@ int sch_ensemble_step(sch_ctx* ctx, int N, int nsteps, const void* m, void* m_ou
     }
     WindowIO<double> io{nsteps, (const double*)m, (double*)m_out, (double*)u_out, (const double*)dW,
                         (const double*)lambda, (const double*)y, nll, logG, iters, status};
+    if (use_pairs(ctx, N, nsteps, 1)) return launch_window_pairs(ctx->ad2, ctx->matern, io, N, S(stream));
     if (ctx->matern) return launch_window_matern<double, 4>(ctx->ad, io, N, S(stream));
     return ctx->ad.solver == SCH_SOLVER_EA ? launch_window<double, 4, SCH_SOLVER_EA>(ctx->ad, io, N, S(stream))
                                            : launch_window<double, 4, SCH_SOLVER_LI>(ctx->ad, io, N, S(stream));
@@ -825,6 +844,7 @@ int jitter_impl(sch_ctx* ctx, int N, int nsteps, int n_iter, double theta, const
     JitterIO<double> io{nsteps, n_iter, 0, theta, tstate, rho, sq, seed, ctr, (const double*)m_start,
                         (double*)dW, (const double*)lambda, (const double*)y, nll, logG, (double*)m_end,
                         (double*)u_end, accepts, iters, status};
+    if (use_pairs(ctx, N, nsteps, 3)) return launch_jitter_pairs(ctx->ad2, ctx->matern, io, N, S(stream));
     if (ctx->matern) return launch_jitter_matern<double, 4>(ctx->ad, io, N, S(stream));
     return ctx->ad.solver == SCH_SOLVER_EA ? launch_jitter<double, 4, SCH_SOLVER_EA>(ctx->ad, io, N, S(stream))
                                            : launch_jitter<double, 4, SCH_SOLVER_LI>(ctx->ad, io, N, S(stream));

@@ -605,7 +605,7 @@ __device__ __forceinline__ void adjoint_load(const ModelArgs<R>& A, Shm<R, TP>* 
         matern_stage_step<R, C>(A, noise, dW, lam, s);
         matern_nodes<R, C, TP>(A, sh, noise, nq);
     } else if constexpr (sizeof(R) == 8) {
-        noise_nodes_centred(A, noise + s * A.K, s0, c0, nq);
+        noise_nodes_centred<C>(A, noise + s * A.K, s0, c0, nq);
     } else {
         noise_nodes<R, C>(A, noise + s * A.K, s0, c0, nq);
     }

@@ -300,6 +300,11 @@ template <typename R, int C>
 int launch_window_matern(const ModelArgs<R>& A, const WindowIO<R>& io, int N, cudaStream_t st);
 template <typename R, int C>
 int launch_jitter_matern(const ModelArgs<R>& A, const JitterIO<R>& io, int N, cudaStream_t st);
+// FP64 windows and jitters on chunks of two nodes (sch_pairs_f64.cu), linearly implicit solver,
+// either noise model; n = 128, 256.  A: the tables of two-node chunks
+int launch_window_pairs(const ModelArgs<double>& A, int matern, const WindowIO<double>& io, int N, cudaStream_t st);
+int launch_jitter_pairs(const ModelArgs<double>& A, int matern, const JitterIO<double>& io, int N, cudaStream_t st);
+size_t pairs_smem(int n, int Ns, int K, int bufs);
 template <typename R>
 int launch_draw(int N, int Ns, int K, R sqdt, uint64_t seed, uint64_t tag, uint64_t ctr, int particle0, int gen32,
                 R* dW, cudaStream_t st);

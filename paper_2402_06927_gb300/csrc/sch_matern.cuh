@@ -21,7 +21,12 @@ namespace sch {
 // Philox4x32-10 in FP32, Philox4x64-10 in FP64
 template <typename R, int C>
 __device__ __forceinline__ void cell_normals(uint64_t seed, int i0, int s, uint64_t pc, uint64_t ctr, R (&z)[C]) {
-    static_assert(C % 4 == 0, "a chunk covers whole Philox blocks");
+    static_assert(C % 4 == 0 || C == 2, "a chunk covers whole Philox blocks, or half of one");
+    if constexpr (C == 2) {
+        const U64x4 r = philox4x64((uint64_t)(i0 >> 2), (uint64_t)s, pc, ctr, seed, SCH_TAG_PCN);
+        const bool second = i0 & 2;
+        box_muller(second ? r.v2 : r.v0, second ? r.v3 : r.v1, z[0], z[1]);
+    }
 #pragma unroll
     for (int b = 0; b < C / 4; ++b) {
         R zb[4];

@@ -113,10 +113,17 @@ __device__ __forceinline__ void var_local_f(const float (&a)[C], const float (&b
         al[i] = ap;
         ga[i] = gp;
     }
-    const float qF = rcp(b[0] - c[0] * al[1]);
-    fview(sh->pa)[t] = a[0] * qF;
-    fview(sh->pc)[t] = -c[0] * ga[1] * qF;
-    fview(sh->pd)[t] = (d[0] - c[0] * de[1]) * qF;
+    if constexpr (C == 2) {   // no interior: the first row couples the last directly
+        const float qF = rcp(b[0]);
+        fview(sh->pa)[t] = a[0] * qF;
+        fview(sh->pc)[t] = c[0] * qF;
+        fview(sh->pd)[t] = d[0] * qF;
+    } else {
+        const float qF = rcp(b[0] - c[0] * al[1]);
+        fview(sh->pa)[t] = a[0] * qF;
+        fview(sh->pc)[t] = -c[0] * ga[1] * qF;
+        fview(sh->pd)[t] = (d[0] - c[0] * de[1]) * qF;
+    }
 }
 
 // The constant matrix (6/h)(M + alpha^2 K) in float: chunk sweep, reduced rows to shared memory
@@ -261,22 +268,30 @@ struct VarReduced {
     }
 };
 
-// SALT increment dU/4 at the six nodes i0 - 1 .. i0 + 4 of a four-node chunk about its
+// SALT increment dU/4 at the nodes i0 - 1 .. i0 + C of a chunk of C = 4 or 2 nodes about its
 // centre theta_c: at theta_c +- d harmonic j gives cos(jd) (a S + b C) +- sin(jd) (a C - b S),
-// (S, C) = (sin, cos)(j theta_c), so a harmonic costs 12 FP64 instructions (noise_nodes:
-// 38).  (s0, c0): the angle of node i0 - 1.
+// (S, C) = (sin, cos)(j theta_c), so a harmonic costs a four-node chunk 12 FP64 instructions
+// (noise_nodes: 38).  (s0, c0): the angle of node i0 - 1.
+template <int C>
 __device__ __forceinline__ void noise_nodes_centred(const ModelArgs<double>& A, const double* wq, double s0, double c0,
-                                                    double (&nq)[6]) {
-    const double cd = A.nco[0][2], sd = A.nsi[0][2];
+                                                    double (&nq)[C + 2]) {
+    static_assert(C == 2 || C == 4, "the centre tables hold three offsets");
+    constexpr int H = C / 2 + 1;
+    const double cd = A.nco[0][H - 1], sd = A.nsi[0][H - 1];
     const double s1 = s0 * cd + c0 * sd, c1 = c0 * cd - s0 * sd;
     const double twoc = 2.0 * c1;
     double sj = s1, cj = c1, sjm = 0.0, cjm = 1.0;
-    double E[3] = {0.0, 0.0, 0.0}, O[3] = {0.0, 0.0, 0.0};
+    double E[H], O[H];
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+        E[k] = 0.0;
+        O[k] = 0.0;
+    }
     for (int j = 0; j < A.K2; ++j) {
         const double a = wq[2 * j], b = wq[2 * j + 1];
         const double v = a * sj + b * cj, q = a * cj - b * sj;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
+        for (int k = 0; k < H; ++k) {
             E[k] += v * A.nco[j][k];
             O[k] += q * A.nsi[j][k];
         }
@@ -287,9 +302,9 @@ __device__ __forceinline__ void noise_nodes_centred(const ModelArgs<double>& A, 
         cj = cn2;
     }
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        nq[3 + k] = E[k] + O[k];
-        nq[2 - k] = E[k] - O[k];
+    for (int k = 0; k < H; ++k) {
+        nq[H + k] = E[k] + O[k];
+        nq[H - 1 - k] = E[k] - O[k];
     }
 }
 
@@ -305,7 +320,6 @@ template <int C, int TP, int NZ>
 __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm<double, TP>* sh,
                                                  Field<double, C>& f, const double* wq, double s0, double c0,
                                                  int& iters, int& flags) {
-    static_assert(C == 4, "the chunk's centre tables are for four nodes");
     const int t = threadIdx.x;
     double W0[C], W0p, W0n;
     {
@@ -313,7 +327,7 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
         if constexpr (NZ == SCH_NOISE_MATERN)
             matern_nodes<double, C, TP>(A, sh, wq, nq);
         else
-            noise_nodes_centred(A, wq, s0, c0, nq);
+            noise_nodes_centred<C>(A, wq, s0, c0, nq);
 #pragma unroll
         for (int i = 0; i < C; ++i) W0[i] = A.dt8 * f.u[i] + nq[i + 1];
         W0p = A.dt8 * f.up + nq[0];

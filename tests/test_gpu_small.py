@@ -2,7 +2,10 @@
 
 * tempering: the float location of the root and its FP64 Newton finish, at dead particles
   (infinite phi), two-valued phi, roots many octaves below the remaining step, and
-  particle counts at the edges of a thread's share.
+  particle counts at the edges of a thread's share;
+* FP64 windows and jitters of small launches (two-node chunks) against the same particles in a
+  launch large enough for four-node chunks: both iterate to 1e-13, so a window of a few
+  steps agrees to 1e-11 and the Metropolis decisions are the same.
 """
 import numpy as np
 import pytest
@@ -10,7 +13,8 @@ import torch
 
 from oracle import filter as OF
 from paper_2402_06927_gb300 import api
-from tests.helpers import tdev
+from workloads import get_config, random_obs, random_state
+from tests.helpers import oracle_model, rel_err, tdev
 
 pytestmark = pytest.mark.gpu
 
@@ -37,3 +41,30 @@ def test_temper_root_matches_oracle(N, kind, frac):
     assert abs(out[1].item() - e) <= 1e-9 * e
     assert out[1].item() >= frac * N * (1 - 1e-12) or out[0].item() == 0.75 * 2.0 ** -60
     assert np.max(np.abs(w.cpu().numpy() - wb)) <= 1e-9 * np.max(wb)
+
+
+@pytest.mark.parametrize("noise", ["modes", "matern"])
+@pytest.mark.parametrize("n", [128, 256])
+def test_two_node_chunks_match_four(n, noise):
+    cfg = get_config("cfg1_f64", n=n)
+    kw = dict(noise=noise, kappa=1.0, eta=0.5) if noise == "matern" else {}
+    g = api.SchModel(L=cfg.L, n=n, alpha=cfg.alpha, mu=cfg.mu, dt=cfg.dt,
+                     amps=[0.05 / j for j in range(1, cfg.K // 2 + 1)], M=cfg.M, sigma=cfg.sigma, tol=1e-13,
+                     max_iter=60, dtype="f64", **kw)
+    om = oracle_model(cfg)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    N, big = 5, 3 * sms + 1
+    m = tdev(np.stack([om.m_from_u(u) for u in random_state(cfg, N, 3)]), g.dtype)
+    y = tdev(random_obs(cfg, 8), g.dtype)
+    dW = g.draw_increments(N, 4, 3, 1, 0)
+    rep = -(-big // N)
+    outs = []
+    for r in (1, rep):
+        ms, ws = m.repeat(r, 1), dW.repeat(r, 1, 1)
+        st = g.ensemble_step(ms, ws, None, y)
+        acc, _, _ = g.jitter(ms, ws, None, y, st["nll"], st["logG"], st["m"], st["u"], 0.3, 0.9, 4, 5, 0)
+        torch.cuda.synchronize()
+        outs.append([v[:N].cpu().numpy() for v in (st["m"], st["u"], ws, st["nll"], acc, st["status"])])
+    for a, b in zip(outs[0][:4], outs[1][:4]):
+        assert rel_err(a, b) < 1e-11
+    assert np.array_equal(outs[0][4], outs[1][4]) and np.array_equal(outs[0][5], outs[1][5])
