@@ -373,6 +373,8 @@ int pf_mala_accept(sch_ctx* ctx, int N, int nsteps, double theta, double h, uint
  * from bufs_a to bufs_b, then pf_jitter_dev (jitter counter stage counter x
  * n_jitter; n_jitter = 0 jitters nothing, which with a tiny ess_min is the bootstrap
  * filter).  A stage reached at temperature one does nothing but copy the rows.
+ * Between a stage's gather and the next one's, its jitter may use the copy of dW that was
+ * gathered from as scratch (the FP64 Matern noise does).
  * bufs_a[PF_STAGE_ARRAYS], bufs_b[PF_STAGE_ARRAYS]: device pointers in the order
  * PF_M_START, PF_M_END, PF_U_END, PF_DW, PF_NLL, PF_LOGG, PF_LAMBDA (the last may be
  * NULL in both); every stage gathers a -> b and swaps the roles, so after n_stages

@@ -813,7 +813,7 @@ namespace {
 int jitter_impl(sch_ctx* ctx, int N, int nsteps, int n_iter, double theta, const double* tstate, double rho,
                 uint64_t seed, uint64_t ctr, const void* m_start, void* dW, const void* lambda, const void* y,
                 double* nll, double* logG, void* m_end, void* u_end, int32_t* accepts, int32_t* iters,
-                int32_t* status, void* stream) {
+                int32_t* status, void* alt, void* stream) {
     if (!ctx || N < 0 || nsteps <= 0 || n_iter < 0) return SCH_ERR_ARG;
     if (!(rho >= 0.0 && rho <= 1.0) || !(theta >= 0.0 && theta <= 1.0)) return SCH_ERR_ARG;
     if (N == 0 || n_iter == 0) return SCH_OK;
@@ -844,6 +844,7 @@ int jitter_impl(sch_ctx* ctx, int N, int nsteps, int n_iter, double theta, const
     JitterIO<double> io{nsteps, n_iter, 0, theta, tstate, rho, sq, seed, ctr, (const double*)m_start,
                         (double*)dW, (const double*)lambda, (const double*)y, nll, logG, (double*)m_end,
                         (double*)u_end, accepts, iters, status};
+    io.alt = (double*)alt;
     if (use_pairs(ctx, N, nsteps, 3)) return launch_jitter_pairs(ctx->ad2, ctx->matern, io, N, S(stream));
     if (ctx->matern) return launch_jitter_matern<double, 4>(ctx->ad, io, N, S(stream));
     return ctx->ad.solver == SCH_SOLVER_EA ? launch_jitter<double, 4, SCH_SOLVER_EA>(ctx->ad, io, N, S(stream))
@@ -870,7 +871,7 @@ int pf_jitter(sch_ctx* ctx, int N, int nsteps, int n_iter, double theta, double 
               double* logG, void* m_end, void* u_end, int32_t* accepts, int32_t* iters, int32_t* status,
               void* stream) {
     return jitter_impl(ctx, N, nsteps, n_iter, theta, nullptr, rho, seed, ctr, m_start, dW, lambda, y, nll, logG,
-                       m_end, u_end, accepts, iters, status, stream);
+                       m_end, u_end, accepts, iters, status, nullptr, stream);
 }
 
 int pf_jitter_dev(sch_ctx* ctx, int N, int nsteps, int n_iter, const double* tstate, double rho, uint64_t seed,
@@ -879,7 +880,7 @@ int pf_jitter_dev(sch_ctx* ctx, int N, int nsteps, int n_iter, const double* tst
                   void* stream) {
     if (!tstate) return SCH_ERR_ARG;
     return jitter_impl(ctx, N, nsteps, n_iter, 0.0, tstate, rho, seed, ctr, m_start, dW, lambda, y, nll, logG,
-                       m_end, u_end, accepts, iters, status, stream);
+                       m_end, u_end, accepts, iters, status, nullptr, stream);
 }
 
 int pf_gated_stages(sch_ctx* ctx, int N, int nsteps, int n_stages, int first_stage, double ess_min, int mode,
@@ -929,9 +930,10 @@ int pf_gated_stages(sch_ctx* ctx, int N, int nsteps, int n_stages, int first_sta
             nxt[a] = t;
         }
         if (events && events[2 * k]) cudaEventRecord((cudaEvent_t)events[2 * k], st);
-        rc = pf_jitter_dev(ctx, N, nsteps, n_jitter, out, rho, seed, stage_ctr * (uint64_t)n_jitter, cur[PF_M_START],
-                           cur[PF_DW], cur[PF_LAMBDA], y, (double*)cur[PF_NLL], (double*)cur[PF_LOGG], cur[PF_M_END],
-                           cur[PF_U_END], accepts, iters ? iters + (size_t)k * N : nullptr, status, stream);
+        // the increments' other copy was gathered from and is free until the next stage's gather
+        rc = jitter_impl(ctx, N, nsteps, n_jitter, 0.0, out, rho, seed, stage_ctr * (uint64_t)n_jitter, cur[PF_M_START],
+                         cur[PF_DW], cur[PF_LAMBDA], y, (double*)cur[PF_NLL], (double*)cur[PF_LOGG], cur[PF_M_END],
+                         cur[PF_U_END], accepts, iters ? iters + (size_t)k * N : nullptr, status, nxt[PF_DW], stream);
         if (rc != SCH_OK) return rc;
         if (events && events[2 * k + 1]) cudaEventRecord((cudaEvent_t)events[2 * k + 1], st);
     }

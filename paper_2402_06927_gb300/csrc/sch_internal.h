@@ -214,6 +214,9 @@ struct JitterIO {
     // previous proposal, [N][Ns][n] in the kernel's register order; null: every proposal
     // starts its Picard iterations from the step's start state
     R* guess = nullptr;
+    // optional (FP64 Matern kernels): scratch of dW's shape.  A proposal's increments are left there
+    // as its pass forms them and an acceptance swaps the two, instead of drawing them again
+    R* alt = nullptr;
 };
 
 template <typename R>

@@ -101,7 +101,15 @@ __global__ void __launch_bounds__(TP, Occ<R, TP>::minb) matern_jitter_kernel(Mod
     const int p = blockIdx.x;
     const int Ns = io.Ns, n = A.n;
     const size_t NQ = (size_t)Ns * n;
+    // The current increments, and in FP64 where a proposal's are kept (null: drawn again on
+    // acceptance): the Box-Muller transform takes about a third of a step's FP64 instructions.
+    // A cycle with n = 128, N = 150, six stages, three proposals in five accepted: 4.53 -> 4.2 ms.
+    // (FP32 draws its proposals again: keeping them was faster, but the compiler then rounds
+    // other operations of the window otherwise.)
+    // A thread reads back only cells that it wrote itself.
     R* dW = io.dW + p * NQ;
+    R* alt = nullptr;
+    if constexpr (sizeof(R) == 8) alt = io.alt ? io.alt + p * NQ : nullptr;
     const R* lam = io.lam ? io.lam + p * NQ : nullptr;
     const uint64_t pc = (uint64_t)(io.particle0 + p);
     __shared__ double sh_state[2];
@@ -126,6 +134,7 @@ __global__ void __launch_bounds__(TP, Occ<R, TP>::minb) matern_jitter_kernel(Mod
             for (int i = 0; i < C; ++i) {
                 const size_t q = (size_t)s * n + i0 + i;
                 R v = pcn_value(io.rho, dW[q], sq, z[i]);
+                if (alt) alt[q] = v;
                 if (lam) {
                     const R l = lam[q];
                     gl += (double)l * (double)v + 0.5 * (double)l * (double)l * A.dt_d;
@@ -152,8 +161,13 @@ __global__ void __launch_bounds__(TP, Occ<R, TP>::minb) matern_jitter_kernel(Mod
         }
         __syncthreads();
         if (sh_acc) {
-            // store the accepted proposal: each thread rewrites its own cells of every step
-            for (int s = 0; s < Ns; ++s) {
+            // the accepted proposal: the other buffer, or each thread rewrites its own cells of every step
+            if (alt) {
+                R* t = dW;
+                dW = alt;
+                alt = t;
+            }
+            for (int s = alt ? Ns : 0; s < Ns; ++s) {
                 R z[C];
                 cell_normals<R, C>(io.seed, i0, s, pc, ctr, z);
 #pragma unroll
@@ -171,6 +185,11 @@ __global__ void __launch_bounds__(TP, Occ<R, TP>::minb) matern_jitter_kernel(Mod
         }
         flags |= fl;
         __syncthreads();
+    }
+    if (dW != io.dW + p * NQ) {
+        for (int s = 0; s < Ns; ++s)
+#pragma unroll
+            for (int i = 0; i < C; ++i) alt[(size_t)s * n + i0 + i] = dW[(size_t)s * n + i0 + i];
     }
     if (threadIdx.x == 0) {
         io.nll[p] = sh_state[0];

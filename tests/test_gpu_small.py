@@ -5,7 +5,9 @@
   particle counts at the edges of a thread's share;
 * FP64 windows and jitters of small launches (two-node chunks) against the same particles in a
   launch large enough for four-node chunks: both iterate to 1e-13, so a window of a few
-  steps agrees to 1e-11 and the Metropolis decisions are the same.
+  steps agrees to 1e-11 and the Metropolis decisions are the same;
+* Matern jitters in gated stages (in FP64 they keep a proposal's increments) against stage by
+  stage (drawn again on acceptance): the same bits.
 """
 import numpy as np
 import pytest
@@ -13,6 +15,7 @@ import torch
 
 from oracle import filter as OF
 from paper_2402_06927_gb300 import api
+from paper_2402_06927_gb300.filter import EnsembleFilter
 from workloads import get_config, random_obs, random_state
 from tests.helpers import oracle_model, rel_err, tdev
 
@@ -68,3 +71,20 @@ def test_two_node_chunks_match_four(n, noise):
     for a, b in zip(outs[0][:4], outs[1][:4]):
         assert rel_err(a, b) < 1e-11
     assert np.array_equal(outs[0][4], outs[1][4]) and np.array_equal(outs[0][5], outs[1][5])
+
+
+@pytest.mark.parametrize("dtype,n,N", [("f32", 256, 40), ("f32", 1024, 24), ("f64", 128, 24), ("f64", 1024, 12)])
+def test_matern_kept_proposals_equal_redrawn(dtype, n, N):
+    g = api.SchModel(L=40.0, n=n, alpha=1.0, mu=0.02, dt=0.025, amps=[0.05], M=16, sigma=0.05,
+                     tol=1e-6 if dtype == "f32" else 1e-13, max_iter=60, dtype=dtype, noise="matern", kappa=1.0,
+                     eta=0.2)
+    u0 = torch.linspace(0, 2 * np.pi, n + 1, device="cuda", dtype=torch.float64)[:-1].sin().mul(0.2).to(g.dtype)
+    m0, _ = g.prior_sample(N, u0.contiguous(), 4, 0.1)
+    y = g.synth_obs(u0.contiguous(), 20, 1)
+    fs = [EnsembleFilter(g, N, 4, 0.5 * N, 0.9, 3, 11, eager_stages=e) for e in (2, 0)]
+    for c in range(2):
+        for f in fs:
+            f.set_state(m0)
+            f.cycle(y, c)
+        for name in ("m_start", "m_end", "u_end", "dW", "nll", "logG", "accepts"):
+            assert torch.equal(getattr(fs[0], name), getattr(fs[1], name)), name
