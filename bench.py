@@ -1024,7 +1024,7 @@ def run_proposal(args):
         "adam_ms": 1e3 * ta,
         "fp32_check_path": {"forward_ms": 1e3 * tf32, "backward_ms": 1e3 * tb32,
                             "forward_tflops": fwd / tf32 / 1e12, "forward_frac_of_fp32_peak": fwd / tf32 / 1e12 / f32_peak},
-        "roofline": {"bound": "tensor", "kernel": "hgemm_kernel (nn_forward, BF16 mma.sync m16n8k16, FP32 accumulation)",
+        "roofline": {"bound": "tensor", "kernel": "conv_tc5_kernel (nn_forward, BF16 tcgen05.mma, FP32 accumulation)",
                      "achieved": fwd / tf / 1e12, "peak": bf_peak, "unit": "TFLOP/s", "frac": fwd / tf / 1e12 / bf_peak,
                      "traffic": None, "peak_note": "measured cuBLAS BF16 burst (MEASURED_PEAKS.json bf16_tflops)"},
         "cpu_baseline": {"value": 1.0 / tho_f, "unit": "samples/s", "cores": 1, "kind": "oracle",

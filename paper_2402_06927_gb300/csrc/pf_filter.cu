@@ -27,9 +27,9 @@ constexpr int RESAMPLE_THREADS = 1024;
 // and any scalar that every warp computes for itself costs as much again.  So the root of
 // ESS(d) = ess_min is located in float first (eight points an evaluation, the exponentials
 // on the special-function unit), two or three Newton steps in FP64 finish it, and only
-// warp 0 sums the partials and takes the decisions.  Tempering, resampling and gathers of 8001
-// particles of n = 1024: 207 us with an Illinois search of 12 to 15 FP64 evaluations summed by
-// every warp, 110 us so.
+// warp 0 sums the partials and takes the decisions.  A searching call at N = 8001 takes 50 us
+// (153 with an Illinois search of 12 to 15 FP64 evaluations summed by every warp), at N = 1024
+// about 26 (62).
 constexpr int TEMPER_POINTS = 8;
 struct TemperShm {
     double dpart[2][8][2];                       // [parity][warp] S1, S2 of an FP64 evaluation
