@@ -392,10 +392,24 @@ __global__ void __cluster_dims__(TEMPER_CTAS, 1, 1) __launch_bounds__(TPT)
     cl.sync();   // no CTA leaves while another may still read its shared memory
 }
 
+// floor(w 2^50) of a weight 0 <= w <= 1, from its bits (anything else as the conversion gives it)
+__device__ __forceinline__ unsigned long long weight_q50(double w) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(w);
+    const int e = (int)(b >> 52);                         // sign and exponent
+    if (e > 1023) return __double2ull_rd(w * 0x1.0p50);   // above 1 + 2^-52, negative, infinite or NaN
+    const int sh = 1025 - e;
+    return (e == 0 || sh > 63) ? 0ull : ((b & 0xfffffffffffffull) | 0x10000000000000ull) >> sh;
+}
+
 // Offspring indices of systematic resampling on integers:
 // q_i = floor(wbar_i 2^50), C = inclusive scan, T = C_{N-1},
 // slot i -> smallest j with C_j > t_i = (i T + floor(U T / 2^53)) / N
 // (equal to floor((i 2^53 + U) T / (N 2^53)) since 2^53 divides i 2^53 T).
+// One CTA, bound by latency and by what each thread does for its N / 1024 weights: q_i is
+// cut out of the weight's bits (a product and a conversion hold the FP64 unit for 64 cycles a
+// warp each), a thread's share is odd so that a warp's shared accesses fall into different
+// banks, and t_i = i (T / N) + V / N + (i (T mod N) + V mod N) / N, V = floor(U T / 2^53),
+// leaves a 32-bit division a slot.  N = 8001: 23 us before, 16 us so.
 __global__ void __launch_bounds__(RESAMPLE_THREADS) resample_kernel(int N, const double* __restrict__ wbar,
                                                                     uint64_t seed, uint64_t stage_ctr,
                                                                     const double* __restrict__ gate,
@@ -408,13 +422,12 @@ __global__ void __launch_bounds__(RESAMPLE_THREADS) resample_kernel(int N, const
         for (int i = t; i < N; i += blockDim.x) idx[i] = i;
         return;
     }
-    const int per = (N + RESAMPLE_THREADS - 1) / RESAMPLE_THREADS;
+    const int per = (N + RESAMPLE_THREADS - 1) / RESAMPLE_THREADS | 1;
     const int beg = t * per;
     const int end = min(N, beg + per);
     unsigned long long loc = 0;
     for (int i = beg; i < end; ++i) {
-        const unsigned long long q = __double2ull_rd(wbar[i] * 0x1.0p50);
-        loc += q;
+        loc += weight_q50(wbar[i]);
         Cs[i] = loc;
     }
     // exclusive scan of per-thread totals
@@ -444,8 +457,10 @@ __global__ void __launch_bounds__(RESAMPLE_THREADS) resample_kernel(int N, const
     const unsigned long long U = r.v0 >> 11;
     const unsigned long long ut_hi = __umul64hi(U, T), ut_lo = U * T;
     const unsigned long long ut53 = (ut_hi << 11) | (ut_lo >> 53);
+    const unsigned long long qT = T / (unsigned)N, qV = ut53 / (unsigned)N;
+    const unsigned rT = (unsigned)(T - qT * (unsigned)N), rV = (unsigned)(ut53 - qV * (unsigned)N);
     for (int i = t; i < N; i += blockDim.x) {
-        const unsigned long long thr = ((unsigned long long)i * T + ut53) / (unsigned long long)N;
+        const unsigned long long thr = (unsigned)i * qT + qV + ((unsigned)i * rT + rV) / (unsigned)N;
         int lo = 0, hi = N - 1;   // smallest j with C_j > thr (C_{N-1} = T > thr)
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;

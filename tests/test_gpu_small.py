@@ -3,6 +3,8 @@
 * tempering: the float location of the root and its FP64 Newton finish, at dead particles
   (infinite phi), two-valued phi, roots many octaves below the remaining step, and
   particle counts at the edges of a thread's share;
+* resampling: weights at the ends of the quantisation (one, zero, subnormal, below 2^-50) and
+  counts at the edges of a thread's share: the oracle's indices;
 * FP64 windows and jitters of small launches (two-node chunks) against the same particles in a
   launch large enough for four-node chunks: both iterate to 1e-13, so a window of a few
   steps agrees to 1e-11 and the Metropolis decisions are the same;
@@ -44,6 +46,26 @@ def test_temper_root_matches_oracle(N, kind, frac):
     assert abs(out[1].item() - e) <= 1e-9 * e
     assert out[1].item() >= frac * N * (1 - 1e-12) or out[0].item() == 0.75 * 2.0 ** -60
     assert np.max(np.abs(w.cpu().numpy() - wb)) <= 1e-9 * np.max(wb)
+
+
+@pytest.mark.parametrize("N", [1, 2, 1023, 1024, 1025, 2049, 8191, 8192])
+@pytest.mark.parametrize("kind", ["one", "equal", "tiny", "spread"])
+def test_resample_indices_match_oracle(N, kind):
+    rng = np.random.default_rng(N)
+    w = np.full(N, 1.0 / N)
+    if kind == "one":
+        w = np.zeros(N)
+        w[N // 3] = 1.0
+    elif kind == "tiny":
+        w[::2] = rng.choice([0.0, 5e-324, 2.0 ** -51, 2.0 ** -50, 3.0 * 2.0 ** -51], w[::2].size)
+        w[0] = 0.5
+    elif kind == "spread":
+        w = np.exp(-rng.gamma(2.0, 5.0, N))
+    w = w / w.sum()
+    for ctr in (0, 77):
+        idx = api.pf_resample(tdev(w, torch.float64), 5, ctr)
+        torch.cuda.synchronize()
+        assert np.array_equal(idx.cpu().numpy(), OF.systematic_resample(w, OF.resample_offset(5, ctr)))
 
 
 @pytest.mark.parametrize("noise", ["modes", "matern"])
