@@ -488,7 +488,10 @@ size_t nn_param_count(const nn_shape* shape);
 /* Workspace bytes for a batch of B samples (activations and gradients). */
 size_t nn_workspace_bytes(const nn_shape* shape, int B);
 /* lambda_out float [B][Ns][K] for u_start float [B][n] and observations y float
- * [B][M] with row stride y_stride floats (0: one y shared by the batch). */
+ * [B][M] with row stride y_stride floats (0: one y shared by the batch).
+ * With NN_BF16, C = 64 and n a multiple of 1024 the convolutions' warps wait for one
+ * another; a wait has a limit (200000 tries), and should one ever reach it, lambda_out
+ * is NaN throughout (the call itself has returned SCH_OK by then). */
 int nn_forward(const nn_shape* shape, int B, const float* params, const float* u_start, const float* y,
                int y_stride, float* lambda_out, void* ws, size_t ws_bytes, void* stream);
 /* Loss L = 1/(2B) sum (lambda - target)^2 (double, device scalar) and its

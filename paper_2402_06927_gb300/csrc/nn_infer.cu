@@ -48,7 +48,12 @@ template <bool FIRST>
 constexpr int NPW = FIRST ? 16 : 8;          // producer warps
 template <bool FIRST>
 constexpr int T5 = 32 * (EPW + NPW<FIRST> + 2);
-constexpr int WAIT_LIMIT = 200000;
+// tries of a wait before it gives up; a build with a low limit runs into it
+#ifndef SCH_CONV_WAIT_LIMIT
+#define SCH_CONV_WAIT_LIMIT 200000
+#endif
+constexpr int WAIT_LIMIT = SCH_CONV_WAIT_LIMIT;
+constexpr int DRAIN_LIMIT = 200000;          // the same for the MMAs in flight at a CTA's end
 
 __device__ __forceinline__ unsigned s2u(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bar_init(uint64_t* b, int n) {
@@ -57,18 +62,21 @@ __device__ __forceinline__ void bar_init(uint64_t* b, int n) {
 __device__ __forceinline__ void bar_arrive(uint64_t* b) {
     asm volatile("mbarrier.arrive.shared.b64 _, [%0];" ::"r"(s2u(b)) : "memory");
 }
+__device__ __forceinline__ bool bar_try(uint64_t* b, int parity) {
+    unsigned done;
+    asm volatile("{.reg .pred p; mbarrier.try_wait.parity.shared.b64 p, [%1], %2; selp.u32 %0, 1, 0, p;}"
+                 : "=r"(done)
+                 : "r"(s2u(b)), "r"(parity)
+                 : "memory");
+    return done;
+}
 // waits for the phase of this parity; false after WAIT_LIMIT tries, or once another wait gave up.
 // Every lane polls, and a warp that goes on to an .aligned tcgen05 instruction takes its decision by
 // a vote: with lane 0 polling for its warp and a shuffle of the answer the branch is no longer
 // provably uniform, and a build of that form faulted.
 __device__ __forceinline__ bool bar_wait(uint64_t* b, int parity, volatile int* gave_up) {
     for (int i = 0; i < WAIT_LIMIT; ++i) {
-        unsigned done;
-        asm volatile("{.reg .pred p; mbarrier.try_wait.parity.shared.b64 p, [%1], %2; selp.u32 %0, 1, 0, p;}"
-                     : "=r"(done)
-                     : "r"(s2u(b)), "r"(parity)
-                     : "memory");
-        if (done) return true;
+        if (bar_try(b, parity)) return true;
         if ((i & 1023) == 1023 && *gave_up) return false;
     }
     *gave_up = 1;
@@ -97,7 +105,7 @@ struct Conv5Args {
 };
 
 struct Conv5Smem {
-    uint64_t full[ST5], ready[ST5], empty[ST5], tfull[2], tempty[2];
+    uint64_t full[ST5], ready[ST5], empty[ST5], tfull[2], tempty[2], drained;
     uint32_t tmem;
     int gave_up;
     alignas(16) float bias[CI];
@@ -130,6 +138,7 @@ __global__ void __launch_bounds__(T5<FIRST>, 1) conv_tc5_kernel(Conv5Args g) {
             bar_init(&sh->tfull[i], 1);
             bar_init(&sh->tempty[i], 128);
         }
+        bar_init(&sh->drained, 1);
         sh->gave_up = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -315,6 +324,16 @@ __global__ void __launch_bounds__(T5<FIRST>, 1) conv_tc5_kernel(Conv5Args g) {
             }
             __syncwarp();
         }
+        // The accumulators are freed and the shared memory given back only after every MMA issued,
+        // also when a wait gave up and no epilogue waits for their commits any more.
+        if (one)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             s2u(&sh->drained))
+                         : "memory");
+        __syncwarp();
+        bool ended = false;
+        for (int i = 0; i < DRAIN_LIMIT && !ended; ++i) ended = bar_try(&sh->drained, 0);
+        if (!__all_sync(FULL, ended)) *gave_up = 1;
     } else if (warp == EPW + NP + 1) {
         // ------------------------------------------------------------------ relay
         // orders the producers' writes, seen through `full`, before the MMAs' reads.  A warp of its
