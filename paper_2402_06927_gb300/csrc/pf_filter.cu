@@ -328,14 +328,19 @@ __global__ void __cluster_dims__(TEMPER_CTAS, 1, 1) __launch_bounds__(TPT)
                 const bool pass = num >= 0.0;
                 // g / |g'| = (num / S2) / (ESS |dlog ESS|): the root is at c + dl
                 const float s1f = (float)S1, s2f = (float)S2;
-                const float dl = (float)num / (2.f * s1f * s1f * (T1 / s1f - T2 / s2f));
+                const float m1 = T1 / s1f, slope = m1 - T2 / s2f;
+                const float dl = (float)num / (2.f * s1f * s1f * slope);
+                // On a plateau of the ESS the float slope is the difference of two nearly equal
+                // means (each right to about 1e-6) and may even have the wrong sign: then dl says
+                // nothing, and the search goes on by midpoints to the narrow bracket
+                const bool steep = slope > 1e-5f * m1;
                 const float cf = (float)c;
                 int act = TEMPER_EVAL;
                 if (pass) {
                     lo = c;
                     ks1 = S1;
                     ks2 = S2;
-                    if (dl <= cf * 0x1p-49f) act = TEMPER_DONE;
+                    if (steep && dl <= cf * 0x1p-49f) act = TEMPER_DONE;
                 } else {
                     hi = c;
                 }
@@ -349,7 +354,7 @@ __global__ void __cluster_dims__(TEMPER_CTAS, 1, 1) __launch_bounds__(TPT)
                 } else {
                     cn = c + (double)dl;
                     if (fabsf(dl) < cf * 0x1p-30f) cn = fma(c, -0x1.0p-51, cn);
-                    if (!(cn > lo && cn < hi) || it % 6 == 0) cn = 0.5 * (lo + hi);
+                    if (!steep || !(cn > lo && cn < hi) || it % 6 == 0) cn = 0.5 * (lo + hi);
                 }
                 if (threadIdx.x == 0) {
                     sh->c = cn;
