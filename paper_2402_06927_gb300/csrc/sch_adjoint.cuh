@@ -214,6 +214,7 @@ __device__ __forceinline__ bool adjoint_step_refined(const ModelArgs<double>& A,
                                                      int& iters) {
     const int t = threadIdx.x;
     constexpr int NW = TP / 32;
+    if (t == 0) sh->nan = 0;
     // w = dv / 4 and S_i = mbar_i + mbar_{i+1} (S[0]: i = -1)
     double w[C + 2], S[C + 1];
     w[0] = A.dt8 * (st.u0p + st.u1p) + nq[0];
@@ -378,7 +379,7 @@ __device__ __forceinline__ bool adjoint_step_refined(const ModelArgs<double>& A,
             const float pm = warp_max_bits((t < NW) ? fview(sh->wred[1])[t] : 0.0f);
             if (t == 0) {
                 int fl = 0;
-                if (!(dm < INFINITY) || !(pm < INFINITY)) fl = FLAG_NONFINITE;
+                if (!(dm < INFINITY) || !(pm < INFINITY) || sh->nan) fl = FLAG_NONFINITE;
                 else if (dm <= A.tolf * pm) fl = FLAG_CONVERGED;
                 sh->flag = fl;
             }

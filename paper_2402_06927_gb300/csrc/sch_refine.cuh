@@ -126,7 +126,9 @@ __device__ __forceinline__ void var_local_f(const float (&a)[C], const float (&b
     }
 }
 
-// The constant matrix (6/h)(M + alpha^2 K) in float: chunk sweep, reduced rows to shared memory
+// The constant matrix (6/h)(M + alpha^2 K) in float: chunk sweep, reduced rows to shared memory.
+// A right-hand side out of the float range (NaN, which the change of m or psi need not show) makes
+// a reduced row NaN: noted in sh->nan, which the step's stop test reads.
 template <int C, int TP>
 __device__ __forceinline__ void helm_local_f(const CTab<float>& T, const float (&r)[C], float (&dp)[C],
                                              Shm<double, TP>* sh) {
@@ -138,8 +140,10 @@ __device__ __forceinline__ void helm_local_f(const CTab<float>& T, const float (
     dp[C - 1] = 0.0f;
 #pragma unroll
     for (int i = C - 2; i >= 1; --i) dp[i] = de[i] - T.gam[i] * dp[i + 1];
-    fview(sh->hpd)[threadIdx.x] = (r[0] - T.a * dp[1]) * T.iBF;
+    const float pd = (r[0] - T.a * dp[1]) * T.iBF;
+    fview(sh->hpd)[threadIdx.x] = pd;
     fview(sh->hde)[threadIdx.x] = de[C - 1];
+    if (!(fabsf(pd) + fabsf(de[C - 1]) < INFINITY)) sh->nan = 1;
 }
 
 // Reduced solve of a variable matrix whose interface rows stay the same over several
@@ -321,6 +325,7 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
                                                  Field<double, C>& f, const double* wq, double s0, double c0,
                                                  int& iters, int& flags) {
     const int t = threadIdx.x;
+    if (t == 0) sh->nan = 0;
     double W0[C], W0p, W0n;
     {
         double nq[C + 2];
@@ -433,7 +438,7 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
             const float mm = warp_max_bits((t < NW) ? fview(sh->wred[1])[t] : 0.0f);
             if (t == 0) {
                 int fl = 0;
-                if (!(dm < INFINITY) || !(mm < INFINITY)) fl = FLAG_NONFINITE;
+                if (!(dm < INFINITY) || !(mm < INFINITY) || sh->nan) fl = FLAG_NONFINITE;
                 else if (dm <= A.tolf * fmaxf(1.0f, mm)) fl = FLAG_CONVERGED;
                 sh->flag = fl;
             }
