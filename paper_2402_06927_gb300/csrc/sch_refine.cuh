@@ -32,16 +32,19 @@ namespace sch {
 // double -> float by truncation and float -> double, on the integer pipe (the
 // conversion instructions run on the narrow pipe).  sh: power-of-two scale of the float
 // side as an exponent-field offset, float = 2^(sh / 2^20) double, -1023 <= sh / 2^20 <= 800.
-// Below the float range: zero; above it, infinite or NaN: NaN.
+// Below the float range: zero; above it, infinite or NaN: NaN.  (The scaled exponent field is
+// unsigned: up to 2847 << 20, and a negative one wraps to 3073 << 20 or more.)
 __device__ __forceinline__ float d2f_bits(double x, int sh = 0) {
-    const int hi = __double2hiint(x);
-    const int ah = (hi & 0x7fffffff) + sh;
-    const unsigned t = __funnelshift_l((unsigned)__double2loint(x), (unsigned)(hi + sh), 3) + 0x40000000u;
-    unsigned r = (t & 0x7fffffffu) | ((unsigned)hi & 0x80000000u);
-    if (ah < (897 << 20)) r = 0u;
-    if (ah >= (1151 << 20) || (hi & 0x7ff00000) == 0x7ff00000) r = 0x7fffffffu;
+    const unsigned hi = (unsigned)__double2hiint(x);
+    const unsigned ah = (hi & 0x7fffffffu) + (unsigned)sh;
+    const unsigned t = __funnelshift_l((unsigned)__double2loint(x), hi + (unsigned)sh, 3) + 0x40000000u;
+    unsigned r = (t & 0x7fffffffu) | (hi & 0x80000000u);
+    if (ah < (897u << 20) || ah >= (3073u << 20)) r = 0u;
+    if ((ah >= (1151u << 20) && ah < (3073u << 20)) || (hi & 0x7ff00000u) == 0x7ff00000u) r = 0x7fffffffu;
     return __uint_as_float(r);
 }
+// (A float NaN or infinity gives a finite value: an iteration that meets one in a right-hand side
+// or a change ends without its result.)
 __device__ __forceinline__ double f2d_bits(float x, int sh = 0) {
     const unsigned b = __float_as_uint(x);
     const unsigned ab = b & 0x7fffffffu;
