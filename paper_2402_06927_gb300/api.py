@@ -15,13 +15,15 @@ from . import _lib
 from ._lib import NNShape, SCH_F32, SCH_F64, SchParams, check, lib
 
 
+# addresses as plain numbers: the argument types convert them, and a c_void_p of one's own is an
+# object more a pointer
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ct.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
     s = torch.cuda.current_stream() if stream is None else stream
-    return ct.c_void_p(s.cuda_stream)
+    return s.cuda_stream
 
 
 def _need(t: torch.Tensor, dtype, shape, name):
@@ -29,7 +31,7 @@ def _need(t: torch.Tensor, dtype, shape, name):
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
-    if tuple(t.shape) != tuple(shape):
+    if t.shape != shape:
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
@@ -156,21 +158,31 @@ class SchModel:
         _need(dW, self.dtype, (N, nsteps, self.K), "dW")
         if lam is not None:
             _need(lam, self.dtype, (N, nsteps, self.K), "lambda")
-        m_out = torch.empty_like(m) if m_out is None else m_out
-        u_out = torch.empty_like(m) if u_out is None else u_out
-        _need(m_out, self.dtype, (N, self.n), "m_out")
-        _need(u_out, self.dtype, (N, self.n), "u_out")
+        # what is allocated here needs no check
+        dev = m.device
+        if m_out is None:
+            m_out = torch.empty_like(m)
+        else:
+            _need(m_out, self.dtype, (N, self.n), "m_out")
+        if u_out is None:
+            u_out = torch.empty_like(m)
+        else:
+            _need(u_out, self.dtype, (N, self.n), "u_out")
         if y is not None:
             _need(y, self.dtype, (self.M,), "y")
-            nll = torch.empty(N, dtype=torch.float64, device=m.device) if nll is None else nll
-            logG = torch.empty(N, dtype=torch.float64, device=m.device) if logG is None else logG
-            _need(nll, torch.float64, (N,), "nll")
-            _need(logG, torch.float64, (N,), "logG")
+            if nll is None:
+                nll = torch.empty(N, dtype=torch.float64, device=dev)
+            else:
+                _need(nll, torch.float64, (N,), "nll")
+            if logG is None:
+                logG = torch.empty(N, dtype=torch.float64, device=dev)
+            else:
+                _need(logG, torch.float64, (N,), "logG")
         else:
             nll = logG = None
         if iters is None and want_iters:
-            iters = torch.empty(N, dtype=torch.int32, device=m.device)
-        status = torch.empty(N, dtype=torch.int32, device=m.device) if status is None else status
+            iters = torch.empty(N, dtype=torch.int32, device=dev)
+        status = torch.empty(N, dtype=torch.int32, device=dev) if status is None else status
         check(lib().sch_ensemble_step(self._h, N, nsteps, _ptr(m), _ptr(m_out), _ptr(u_out), _ptr(dW), _ptr(lam),
                                       _ptr(y), _ptr(nll), _ptr(logG), _ptr(iters), _ptr(status), _stream()),
               "sch_ensemble_step")

@@ -33,3 +33,17 @@ def test_one_stage_cycle_dispatches_one_copy():
         st = f.cycle(y, 1)
     assert len(st.stages) == 1
     assert ops.names == ["copy_"]
+
+
+def test_given_outputs_are_checked():
+    """ensemble_step checks the outputs that a caller gives, each by shape, type and layout."""
+    cfg = get_config("cfg2_f32", n=256, M=16)
+    g = gpu_model(cfg)
+    m, dW = torch.zeros(3, 256, device="cuda"), torch.zeros(3, 2, g.K, device="cuda")
+    y = torch.zeros(16, device="cuda")
+    for name, good in (("m_out", m), ("u_out", m), ("nll", m[:, 0].double()), ("logG", m[:, 0].double())):
+        g.ensemble_step(m, dW, None, y, **{name: torch.empty_like(good)})
+        for bad in (torch.empty_like(good)[:2], torch.empty_like(good).half(), torch.empty_like(good).cpu(),
+                    torch.empty((2 * g.n, 3), device="cuda", dtype=good.dtype).t()[:, ::2].squeeze()):
+            with pytest.raises((TypeError, ValueError)):
+                g.ensemble_step(m, dW, None, y, **{name: bad})
