@@ -248,6 +248,7 @@ void fill_refine(const sch_params& p, int C, ModelArgs<double>& A) {
     A.tolf = (float)A.tol;
     A.s6 = 3.0 / h;
     A.kz = p.dt * h / 12.0;
+    A.plain = p.alpha > 2e4 * h;
     for (int j = 0; j < p.K / 2; ++j)
         for (int k = 0; k < 3; ++k) {
             const double d = 2.0 * M_PI * (j + 1) * (k + 0.5) / p.n;
@@ -677,9 +678,10 @@ namespace {
 // chunks (nearly) all have an FP64 unit of their own.  Five steps, four-node against two-node
 // chunks, us (152 SMs): n = 128, N = 304 172 / 132, 456 173 / 155, 608 181 / 182; n = 256, N =
 // 152 172 / 138, 228 182 / 193; n = 512, N = 16 196 / 217 (the reduced solve of 256 rows
-// takes back more than the FP64 unit gives).
+// takes back more than the FP64 unit gives).  The plain iteration stays on four-node chunks: with
+// alpha = 1e6 h its u is 1.4e-5 from the exact one on those, 8.9e-5 on two-node chunks.
 bool use_pairs(const sch_ctx* ctx, int N, int nsteps, int bufs) {
-    if (ctx->p.dtype != SCH_F64 || ctx->ad.solver != SCH_SOLVER_LI || ctx->p.n > 256) return false;
+    if (ctx->p.dtype != SCH_F64 || ctx->ad.solver != SCH_SOLVER_LI || ctx->p.n > 256 || ctx->ad.plain) return false;
     if (N > (ctx->p.n == 128 ? 3 : 1) * device_sms()) return false;
     return ctx->matern || pairs_smem(ctx->p.n, nsteps, ctx->Q, bufs) <= 200 * 1024;
 }

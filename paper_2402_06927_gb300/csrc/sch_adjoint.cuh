@@ -287,7 +287,7 @@ __device__ __forceinline__ bool adjoint_step_refined(const ModelArgs<double>& A,
     for (int r = 0; r < NW; ++r) ge = max(ge, __float_as_uint(fview(sh->wred[0])[r]));
     ge >>= 20;
     const int shq = min(1023 - (int)ge, 800) * (1 << 20);
-    int bad = ge >= 0x7ffu;
+    int bad = ge >= 0x7ffu || A.plain;
     // warp 0: the elimination of the interface rows and the lane system's PCR multipliers
     VarReduced<TP> V;
     if (t < 32) V.factor(fview(sh->ae), fview(sh->ge), fview(sh->pa), fview(sh->pc), fview(sh->sw));

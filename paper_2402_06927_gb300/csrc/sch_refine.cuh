@@ -360,8 +360,8 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
     const double bq = A.b0 - 2.0 * A.c0;
     const double h2 = A.helg;                    // off-diagonal of (6/h)(M + alpha^2 K)
     const float c0f = A.c0f, b0f = A.b0f;
-    int it = 1, bad = 0;
-    for (;; ++it) {
+    int it = 1, bad = A.plain;
+    for (; !bad; ++it) {
         float al[C], ga[C], de[C];
         {
             // w = dv / 4; r_i = D0_i - c0 (m_{i-1} + m_{i+1}) - b0 m_i + w_{i-1} T_{i-1} - w_{i+1} T_i,
@@ -459,10 +459,7 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
         }
         const int fl = sh->flag;
         if (fl & FLAG_CONVERGED) break;
-        if ((fl & FLAG_NONFINITE) || it == A.max_iter) {
-            bad = 1;
-            break;
-        }
+        bad = (fl & FLAG_NONFINITE) || it == A.max_iter;
     }
     if (bad) {
         Field<double, C> g = f;

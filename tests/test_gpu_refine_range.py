@@ -38,6 +38,23 @@ def test_helmholtz_side_out_of_float_range(n):
         assert rel_err(out["u"][p].cpu().numpy(), ref[p][1]) < 1e-11
 
 
+@pytest.mark.parametrize("n", [128, 256])
+def test_extreme_alpha_takes_the_plain_iteration(n):
+    """alpha = 1e6 h, where the float Helmholtz solve is singular: a small launch gives what a large
+    one does (the plain iteration on the same chunks), in the iterations of the oracle."""
+    cfg = get_config("cfg1_f64", n=n)
+    g, om = gpu_model(cfg, alpha=1e6 * cfg.h), oracle_model(cfg)
+    N = 3 * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    m = tdev(np.stack([om.m_from_u(u) for u in random_state(cfg, 4, 3)]), g.dtype)
+    dW = tdev(random_increments(cfg, 4, 4, steps=4), g.dtype)
+    few = g.ensemble_step(m, dW)
+    many = g.ensemble_step(m.repeat(-(-N // 4), 1), dW.repeat(-(-N // 4), 1, 1))
+    torch.cuda.synchronize()
+    for k in ("m", "u", "iters", "status"):
+        assert torch.equal(few[k], many[k][:4]), k
+    assert torch.all(few["status"] == 0) and torch.all(few["iters"] <= 4 * 4)
+
+
 SOURCE = """
 #include "sch_kernels.cuh"
 __global__ void convert(int N, const double* x, const int* sh, unsigned* out, double* back) {
