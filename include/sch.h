@@ -27,6 +27,14 @@
  *  - Sizes: n must equal C * TP with TP a power of two in [32, 512], where
  *    C = 8 for SCH_F32 and C = 4 for SCH_F64 (so n in {256 .. 4096} for f32,
  *    {128 .. 2048} for f64); n % M == 0; K even, 2 <= K <= 64.
+ *  - A particle's results do not depend on the other particles of its launch, but with
+ *    SCH_F64 and the linearly implicit solver sch_ensemble_step and the jitters choose
+ *    how a particle is split over threads by N: n = 128 with N <= 3 SMs (456 on a
+ *    GB300 of 152) and n = 256 with N <= SMs take chunks of two nodes, every other
+ *    launch chunks of four.  The two agree to the stop test's tol and to rounding, not
+ *    bit for bit, and a Metropolis decision within that of its threshold can
+ *    differ: between an ensemble and a part of it launched alone, and between devices
+ *    with other SM counts.  Launches of one N on one device reproduce each other.
  *
  * Random numbers: Philox4x64-10 (Salmon et al., SC'11), key (seed, purpose),
  * counter (block, step, particle, stream counter); normals by Box-Muller on
@@ -465,12 +473,18 @@ int pf_nudge(sch_ctx* ctx, int N, int nsteps, int mode, int max_iter, double gto
  *   F[c][2(j-1)], F[c][2j-1] = (1/P) sum_q h[c][q] sin, cos(2 pi j q / P), P = n/16
  *   lambda = Wh F + bh
  * Parameters are one FP32 vector (per layer w[C][Cin][5], b[C]; then Wh[K Ns][C K],
- * bh[K Ns]); activations and gradients are FP32 in memory.  The contractions
+ * bh[K Ns]); lambda and the parameters' gradients are FP32.  The contractions
  * (every convolution, the mode projection and the head, forward and backward)
  * run in the shape's precision:
- *   NN_FP32  FP32 operands, FP32 accumulation (CUDA cores; the check path);
- *   NN_BF16  operands rounded to BF16, FP32 accumulation (tensor cores,
- *            mma.sync m16n8k16); Adam keeps FP32 master weights.
+ *   NN_FP32  FP32 operands, FP32 accumulation (CUDA cores; the check path), FP32
+ *            activations and activation gradients in memory;
+ *   NN_BF16  operands rounded to BF16, FP32 accumulation on the tensor cores
+ *            (mma.sync m16n8k16; with C = 64 and n a multiple of 1024 the forward
+ *            convolutions after the first on tcgen05.mma).  With C = 64 the
+ *            activations and their gradients are kept as the BF16 values that the
+ *            contractions round them to (nn_forward: n a multiple of 1024; nn_backward:
+ *            n a power of two from 128, K even and at most 64), else as FP32.  Adam
+ *            keeps FP32 master weights.
  * ------------------------------------------------------------------------- */
 enum { NN_FP32 = 0, NN_BF16 = 1 };
 typedef struct {

@@ -4,7 +4,7 @@
 // [Ns][K] (used in place of, or as the starting point of, the optimiser of
 // Sec. 3.1.3; any drift keeps the weights consistent through Girsanov).
 //
-// Network (FP32 parameters and activations, FP32 accumulation):
+// Network (FP32 parameters, FP32 accumulation):
 //   x0[b] = (u_start, (y - u_start(x_obs)) / sigma scattered at the obs nodes)   2 x n
 //   four circular convolutions, kernel 5, stride 2, padding 2, C channels, ReLU  -> C x n/16
 //   Fourier-mode projection F[c][k] = (1/P) sum_q h[c][q] {sin,cos}(2 pi j q / P)
@@ -13,8 +13,10 @@
 // (implicit im2col for the convolutions), so no im2col buffer is formed: a SIMT
 // FP32 kernel (NN_FP32, the check path), or a tensor-core kernel that rounds both
 // operands to BF16 as it stages them in shared memory and accumulates in FP32
-// with mma.sync m16n8k16 (NN_BF16).  Parameters, activations and gradients stay
-// FP32 in memory in both (the FP32 master weights of Adam).
+// with mma.sync m16n8k16 (NN_BF16).  Parameters, activations and gradients are FP32 in
+// memory in both.  The BF16 passes of 64 channels are elsewhere, on BF16 activations:
+// inference with n a multiple of 1024 in nn_infer.cu, training with n a power of two in
+// nn_train.cu.
 #include "nn_internal.h"
 
 namespace sch {

@@ -397,11 +397,11 @@ __global__ void __cluster_dims__(TEMPER_CTAS, 1, 1) __launch_bounds__(TPT)
     cl.sync();   // no CTA leaves while another may still read its shared memory
 }
 
-// floor(w 2^50) of a weight 0 <= w <= 1, from its bits (anything else as the conversion gives it)
+// floor(w 2^50) of a weight 0 <= w < 2, from its bits (anything else as the conversion gives it)
 __device__ __forceinline__ unsigned long long weight_q50(double w) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(w);
     const int e = (int)(b >> 52);                         // sign and exponent
-    if (e > 1023) return __double2ull_rd(w * 0x1.0p50);   // above 1 + 2^-52, negative, infinite or NaN
+    if (e > 1023) return __double2ull_rd(w * 0x1.0p50);   // at least 2, negative, infinite or NaN
     const int sh = 1025 - e;
     return (e == 0 || sh > 63) ? 0ull : ((b & 0xfffffffffffffull) | 0x10000000000000ull) >> sh;
 }

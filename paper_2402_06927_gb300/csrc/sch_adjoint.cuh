@@ -518,17 +518,7 @@ __device__ __forceinline__ void mode_sums_centred(const ModelArgs<double>& A, do
                 cj = cn2;
             }
         }
-        // after the exchanges over 16, 8 and 4 a lane holds sum number (lane >> 2) of the eight
-#pragma unroll
-        for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1)
-#pragma unroll
-            for (int k = 0; k < h; ++k) {
-                const bool up = lane & o;
-                const double keep = up ? v[k + h] : v[k], send = up ? v[k] : v[k + h];
-                v[k] = keep + __shfl_xor_sync(FULL, send, o);
-            }
-        v[0] += __shfl_xor_sync(FULL, v[0], 2);
-        v[0] += __shfl_xor_sync(FULL, v[0], 1);
+        warp_sums8(v);
         const int k = 2 * j0 + (lane >> 2);
         if ((lane & 3) == 0 && k < A.K) red[warp * A.K + k] = v[0];
     }
