@@ -658,6 +658,20 @@ def _adjoint_flops(n, K, N, Ns, it_fwd, it_adj, matern_k=None, solver="li"):
             + n * (ADJ_FLOPS_PER_NODE_ITER * it_adj + (ADJ_FLOPS_PER_NODE_STEP + 2 * mf) * N * Ns))
 
 
+# What the FP64 (linearly implicit) adjoint window executes on the FP64 pipe, instructions a node:
+# most of a defect-corrected iteration runs in float, so the method's flops above do not
+# measure that pipe.  Counted with ncu (smsp__inst_executed_pipe_fp64) at n = 1024 with two
+# tolerances: 20 a forward iteration, 17.25 an adjoint iteration; per step, forward and
+# adjoint together, 39 and 4.6 a mode, or 113 with the Matern noise of three solves (25 a solve).
+FP64_FWD_ITER, FP64_ADJ_ITER, FP64_STEP, FP64_STEP_MODE, FP64_STEP_SOLVE = 20.0, 17.25, 39.0, 4.6, 25.0
+
+
+def _adjoint_fp64_flops(n, K, N, Ns, it_fwd, it_adj, matern_k=None):
+    """FP64 instructions of an adjoint window call, each as the two flops of its issue slot."""
+    step = FP64_STEP + (FP64_STEP_MODE * K if matern_k is None else FP64_STEP_SOLVE * matern_k)
+    return 2.0 * n * (FP64_FWD_ITER * it_fwd + FP64_ADJ_ITER * it_adj + step * N * Ns)
+
+
 def _nudging_config(args, name):
     """The nudging workload, on FP32 fields (EA Picard, tolerance 1e-6) with --f32."""
     from workloads import get_config
@@ -670,7 +684,7 @@ def _precision(args):
         return ("f32", "EA", "float,8,128,EA", fp32_peak_tflops(),
                 f"FP32 FMA pipe {sm_count()} SMs x 128 lanes x 2 x max SM clock")
     return ("f64", "LI", "double,4,256,LI", fp64_peak_tflops(),
-            f"FP64 pipe {sm_count()} SMs x 2 DFMA lanes x 2 x max SM clock")
+            f"FP64 pipe {sm_count()} SMs x 2 DFMA lanes x 2 x max SM clock; achieved: FP64 instructions x 2")
 
 
 def _ckpt_note(ckpt):
@@ -713,8 +727,9 @@ def run_adjoint(args):
     assert int(out["status"].abs().sum().item()) == 0, "adjoint status flags"
     it_fwd = int(fwd["iters"].sum().item())
     it_adj = int(out["iters"].sum().item()) - it_fwd
-    achieved = _adjoint_flops(n, K, N, Ns, it_fwd, it_adj, cfg.matern_k if args.matern else None,
-                              slabel.lower()) / t / 1e12
+    mk = cfg.matern_k if args.matern else None
+    achieved = (_adjoint_flops(n, K, N, Ns, it_fwd, it_adj, mk, "ea") if args.f32
+                else _adjoint_fp64_flops(n, K, N, Ns, it_fwd, it_adj, mk)) / t / 1e12
     cpu = None
     if not args.no_cpu:
         import numpy as np
@@ -811,7 +826,8 @@ def run_mala(args):
     t_acc = _event_time(lambda: g.mala_accept(dWc, dWp, lam, J, Jp, gJ, gJp, None, theta, h, 31, 0), 20, flush)
     it_fwd = int(fwd["iters"].sum().item())
     it_adj = int(adj["iters"].sum().item()) - it_fwd
-    achieved = _adjoint_flops(n, K, N, Ns, it_fwd, it_adj, solver=slabel.lower()) / t_adj / 1e12
+    achieved = (_adjoint_flops(n, K, N, Ns, it_fwd, it_adj, solver="ea") if args.f32
+                else _adjoint_fp64_flops(n, K, N, Ns, it_fwd, it_adj)) / t_adj / 1e12
     cpu = None
     if not args.no_cpu:
         from oracle.model import Model

@@ -204,7 +204,7 @@ __device__ __forceinline__ void adjoint_step(const ModelArgs<R>& A, Shm<R, TP>* 
 // and warp 0's elimination of them are formed once a step and an iteration only runs
 // right-hand sides through them.  The float side is scaled by a power of two that takes
 // max|g| to [1, 2), so a gradient of any size stays in the float range; the stop test is
-// relative and does not see it.  14 FP64 instructions a node and iteration (about 45
+// relative and does not see it.  17 FP64 instructions a node and iteration (about 45
 // before).  Returns false, with g unchanged, when the iteration does not converge or leaves
 // the float range: the caller then runs adjoint_step.
 template <int C, int TP>

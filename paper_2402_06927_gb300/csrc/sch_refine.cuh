@@ -8,14 +8,17 @@
 // quarter of them in that one warp.  Here an iteration forms, in double,
 //   r = (M - mu dt/2 K - 1/2 A_dv) m0 - (M + mu dt/2 K + 1/2 A_dv) m,
 // solves the same variable matrix for the change of m in float, adds it in double, then
-// forms r' = M m - H u and solves for the change of u in the same way: 17 FP64
-// instructions a node and iteration, none in the reduced solves.  The iterates
+// forms r' = M m - H u and solves for the change of u in the same way: 20 FP64
+// instructions a node and iteration (counted with ncu), none in the reduced solves.  The iterates
 // are those of sch_step up to the float solve's relative error (about 1e-7) in each
 // *change*, which the next residual sees and removes, so the sequence contracts as
-// before, stops by the same test after the same number of iterations and ends at the
-// fixed point of the double residuals.  A step whose corrected iteration does not
+// before, stops by the same test after the same number of iterations (a few more where
+// alpha is far below a cell: 108 against 71 over five steps at alpha = h / 20, n = 2048) and ends
+// at the fixed point of the double residuals.  A step whose corrected iteration does not
 // converge, or leaves the float range, is run again from its start by sch_step: its result
-// and its status are those of the plain FP64 iteration.
+// and its status are those of the plain FP64 iteration.  u, no longer solved for anew, is within
+// 1e-13 of H^{-1} M m for alpha up to 1e4 cells (the plain iteration's 1e-9 there); beyond 2e4
+// cells every step is the plain iteration.
 //
 // Measured (one GB300, before -> after): gradients of 256 particles, n = 1024, 20 steps 11.60
 // -> 4.20 ms; a filter cycle with n = 256, N = 32 9.63 -> 3.61 ms, with the Matern noise at
