@@ -557,7 +557,7 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 bool cl_supported(const NNDims& d) {
     // 64 channels; every layer's output a whole number of 64-position tiles
-    return d.prec == NN_BF16 && d.C == CI && d.L[4] % 64 == 0 && d.n <= (1 << 21);
+    return d.prec == NN_BF16 && d.C == CI && d.L[4] % 64 == 0 && d.n <= (1 << 21) && head_count(d) <= HEAD_MAX;
 }
 
 // layers 2..4 and the mode features of the batch, the packed parameters, the failure word

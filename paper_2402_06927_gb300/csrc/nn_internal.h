@@ -39,6 +39,12 @@ inline NNDims make_dims(const nn_shape* s) {
     return d;
 }
 
+// entries of the head's matrix
+inline size_t head_count(const NNDims& d) { return (size_t)d.K * d.Ns * d.C * d.K; }
+// the BF16 passes of 64 channels count the head's entries in 32 bits; a larger head (from 4 GB of
+// FP32 weights) takes the generic pass, which counts in 64
+constexpr size_t HEAD_MAX = (size_t)1 << 30;
+
 constexpr int TM = 64, TN = 64;   // output tile of the generic GEMMs (and of their split-K rule)
 
 // k-splits for a reduction with few output tiles (weight gradients: the sum runs over

@@ -943,7 +943,7 @@ int grid_for(size_t n) { return (int)max((size_t)1, min((n + 255) / 256, (size_t
 bool cf_supported(const NNDims& d) {
     const int P = d.L[4];
     return d.prec == NN_BF16 && d.C == CF_C && P >= 8 && (P & (P - 1)) == 0 && d.n == 16 * P && d.K % 2 == 0 &&
-           d.K <= 64;
+           d.K <= 64 && head_count(d) <= HEAD_MAX;
 }
 
 size_t cf_workspace_bytes(const NNDims& d, int B) { return make_layout(d, B).total; }
