@@ -47,3 +47,14 @@ def test_given_outputs_are_checked():
                     torch.empty((2 * g.n, 3), device="cuda", dtype=good.dtype).t()[:, ::2].squeeze()):
             with pytest.raises((TypeError, ValueError)):
                 g.ensemble_step(m, dW, None, y, **{name: bad})
+
+
+def test_calls_run_on_the_current_stream():
+    """The stream handed to the library is torch's current one: of the context, else the default."""
+    from paper_2402_06927_gb300 import api
+    s = torch.cuda.Stream()
+    assert api._stream() == torch.cuda.current_stream().cuda_stream
+    with torch.cuda.stream(s):
+        assert api._stream() == s.cuda_stream
+    assert api._stream(s) == s.cuda_stream
+    assert api._stream() == torch.cuda.current_stream().cuda_stream
