@@ -99,7 +99,7 @@ JITTER_TRAFFIC_BYTES = {"cfg2_f32": {
     # the same sources with one comment corrected (no code change): the capture above
     "0128ccf827d69e0960f91b1175216b6f6335b443": 4607488,
     # the same kernel code with the FP64 defect correction in the shared headers: 4.607232 MB read
-    "3b0d7d52c799c54b2f416abf548e4626424a6fdd": 4607232,
+    "5480252971492c19e504a17948cf93d5a820904a": 4607232,
 }, "cfg5_f32": {
     # gjitter_kernel<8,2,4,1>, profiles/gjitter_kernel_cfg5_n4096_N8192.md: 148.514304 MB read,
     # 226.438400 MB written
@@ -124,7 +124,7 @@ JITTER_TRAFFIC_BYTES = {"cfg2_f32": {
     # the same sources with one comment corrected (no code change): the capture above
     "e4040ce2ae15928553e68f8ca69e7f19b0e8e742": 14744669952,
     # the same kernel code with the FP64 defect correction in the shared headers: 2.70 GB read, 12.01 GB written
-    "39b4d9ec90719676a2411b0b696032bee4099e5b": 14710000000,
+    "a6ac43127bd913d823342b269b1170136fd0a12d": 14710000000,
 }}
 
 

@@ -233,6 +233,13 @@ void cast_tab(const HTab& s, CTab<R>& d) {
     d.ge = (R)s.ge;
 }
 
+// alpha > 2e4 h: the plain FP64 iteration throughout.  The float Helmholtz solve of the defect
+// correction is then next to singular: at n = 128 a step needs 5 iterations instead of 3 at alpha =
+// 1e4 h, but up to 23 at 5e4 h (the adjoint 47 instead of 6), and at 1e6 h every correction leaves
+// the float range.  (A rule in the host's tables: a branch in the kernels cost their small launches
+// 1 to 4%, and 8% at n = 256, N = 1500.)
+bool plain_only(const sch_params& p) { return p.alpha > 2e4 * p.L / p.n; }
+
 void fill_refine(const sch_params&, int, ModelArgs<float>&) {}
 void fill_refine(const sch_params& p, int C, ModelArgs<double>& A) {
     const double h = p.L / p.n, g = 1.0 - 6.0 * p.alpha * p.alpha / (h * h);
@@ -248,7 +255,7 @@ void fill_refine(const sch_params& p, int C, ModelArgs<double>& A) {
     A.tolf = (float)A.tol;
     A.s6 = 3.0 / h;
     A.kz = p.dt * h / 12.0;
-    A.plain = p.alpha > 2e4 * h;
+    if (plain_only(p)) A.helf.iBF = NAN;   // the first iteration of every step gives up
     for (int j = 0; j < p.K / 2; ++j)
         for (int k = 0; k < 3; ++k) {
             const double d = 2.0 * M_PI * (j + 1) * (k + 0.5) / p.n;
@@ -681,7 +688,7 @@ namespace {
 // takes back more than the FP64 unit gives).  The plain iteration stays on four-node chunks: with
 // alpha = 1e6 h its u is 1.4e-5 from the exact one on those, 8.9e-5 on two-node chunks.
 bool use_pairs(const sch_ctx* ctx, int N, int nsteps, int bufs) {
-    if (ctx->p.dtype != SCH_F64 || ctx->ad.solver != SCH_SOLVER_LI || ctx->p.n > 256 || ctx->ad.plain) return false;
+    if (ctx->p.dtype != SCH_F64 || ctx->ad.solver != SCH_SOLVER_LI || ctx->p.n > 256 || plain_only(ctx->p)) return false;
     if (N > (ctx->p.n == 128 ? 3 : 1) * device_sms()) return false;
     return ctx->matern || pairs_smem(ctx->p.n, nsteps, ctx->Q, bufs) <= 200 * 1024;
 }

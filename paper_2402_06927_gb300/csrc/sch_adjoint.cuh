@@ -214,7 +214,6 @@ __device__ __forceinline__ bool adjoint_step_refined(const ModelArgs<double>& A,
                                                      int& iters) {
     const int t = threadIdx.x;
     constexpr int NW = TP / 32;
-    if (t == 0) sh->nan = 0;
     // w = dv / 4 and S_i = mbar_i + mbar_{i+1} (S[0]: i = -1)
     double w[C + 2], S[C + 1];
     w[0] = A.dt8 * (st.u0p + st.u1p) + nq[0];
@@ -287,7 +286,7 @@ __device__ __forceinline__ bool adjoint_step_refined(const ModelArgs<double>& A,
     for (int r = 0; r < NW; ++r) ge = max(ge, __float_as_uint(fview(sh->wred[0])[r]));
     ge >>= 20;
     const int shq = min(1023 - (int)ge, 800) * (1 << 20);
-    int bad = ge >= 0x7ffu || A.plain;
+    int bad = ge >= 0x7ffu;
     // warp 0: the elimination of the interface rows and the lane system's PCR multipliers
     VarReduced<TP> V;
     if (t < 32) V.factor(fview(sh->ae), fview(sh->ge), fview(sh->pa), fview(sh->pc), fview(sh->sw));
@@ -360,6 +359,7 @@ __device__ __forceinline__ bool adjoint_step_refined(const ModelArgs<double>& A,
         }
         // (6/h)(B^T psi - H z), (B^T x)_i = 1/2 (S_{i-1} x_{i-1} - S_i x_{i+1})
         float dpH[C];
+        bool out;
         {
             float r[C];
 #pragma unroll
@@ -370,16 +370,16 @@ __device__ __forceinline__ bool adjoint_step_refined(const ModelArgs<double>& A,
                 e -= h2 * lap[i];
                 r[i] = d2f_bits(e, shq);
             }
-            helm_local_f<C, TP>(A.helf, r, dpH, sh);
+            out = helm_local_f<C, TP>(A.helf, r, dpH, sh);
         }
-        __syncthreads();                                             // B3
+        const int nan = __syncthreads_or(out);                       // B3
         if (t < 32) {
             warp_solve_const<float, TP>(A.helf, A.rhelf, fview(sh->hpd), fview(sh->hde), fview(sh->hE), fview(sh->hF));
             const float dm = warp_max_bits((t < NW) ? fview(sh->wred[0])[t] : 0.0f);
             const float pm = warp_max_bits((t < NW) ? fview(sh->wred[1])[t] : 0.0f);
             if (t == 0) {
                 int fl = 0;
-                if (!(dm < INFINITY) || !(pm < INFINITY) || sh->nan) fl = FLAG_NONFINITE;
+                if (!(dm < INFINITY) || !(pm < INFINITY) || nan) fl = FLAG_NONFINITE;
                 else if (dm <= A.tolf * pm) fl = FLAG_CONVERGED;
                 sh->flag = fl;
             }

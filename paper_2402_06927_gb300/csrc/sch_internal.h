@@ -70,10 +70,6 @@ struct RefineArgs<double> {
     double s6, kz;        // 3 / h, dt h / 12
     // cos(j d_k), sin(j d_k) for harmonic j + 1 and offsets d_k = (k + 1/2) 2 pi / n
     double nco[SCH_MAX_K / 2][3], nsi[SCH_MAX_K / 2][3];
-    // alpha > 2e4 h: the plain iteration throughout.  The float Helmholtz solve is then next to
-    // singular: at n = 128 a step needs 5 iterations instead of 3 at alpha = 1e4 h, but up to 23 at
-    // 5e4 h (the adjoint 47 instead of 6), and at 1e6 h every correction leaves the float range
-    int plain;
 };
 
 // Precomputed scalars of the discretised model, passed by value to kernels

@@ -48,7 +48,6 @@ struct __align__(16) Shm {
     R wred[2][32];                                       // per-warp convergence maxima
     double dsum[2][32];                                  // per-warp double sums
     int flag;
-    int nan;                                             // a float right-hand side left its range (sch_refine.cuh)
 };
 
 template <typename R, int TP>

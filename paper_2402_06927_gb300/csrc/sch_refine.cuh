@@ -133,10 +133,11 @@ __device__ __forceinline__ void var_local_f(const float (&a)[C], const float (&b
 }
 
 // The constant matrix (6/h)(M + alpha^2 K) in float: chunk sweep, reduced rows to shared memory.
-// A right-hand side out of the float range (NaN, which the change of m or psi need not show) makes
-// a reduced row NaN: noted in sh->nan, which the step's stop test reads.
+// True where a right-hand side is out of the float range (NaN, which the change of m or psi need not
+// show and which makes a reduced row NaN): the barrier that follows takes it to the stop test.  (As a
+// flag in shared memory it cost windows of n = 128 up to 4%, on the barrier nothing that shows.)
 template <int C, int TP>
-__device__ __forceinline__ void helm_local_f(const CTab<float>& T, const float (&r)[C], float (&dp)[C],
+__device__ __forceinline__ bool helm_local_f(const CTab<float>& T, const float (&r)[C], float (&dp)[C],
                                              Shm<double, TP>* sh) {
     float de[C];
     de[0] = 0.0f;
@@ -149,7 +150,7 @@ __device__ __forceinline__ void helm_local_f(const CTab<float>& T, const float (
     const float pd = (r[0] - T.a * dp[1]) * T.iBF;
     fview(sh->hpd)[threadIdx.x] = pd;
     fview(sh->hde)[threadIdx.x] = de[C - 1];
-    if (!(fabsf(pd) + fabsf(de[C - 1]) < INFINITY)) sh->nan = 1;
+    return !(fabsf(pd) + fabsf(de[C - 1]) < INFINITY);
 }
 
 // Reduced solve of a variable matrix whose interface rows stay the same over several
@@ -331,7 +332,6 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
                                                  Field<double, C>& f, const double* wq, double s0, double c0,
                                                  int& iters, int& flags) {
     const int t = threadIdx.x;
-    if (t == 0) sh->nan = 0;
     double W0[C], W0p, W0n;
     {
         double nq[C + 2];
@@ -363,8 +363,8 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
     const double bq = A.b0 - 2.0 * A.c0;
     const double h2 = A.helg;                    // off-diagonal of (6/h)(M + alpha^2 K)
     const float c0f = A.c0f, b0f = A.b0f;
-    int it = 1, bad = A.plain;
-    for (; !bad; ++it) {
+    int it = 1, bad = 0;
+    for (;; ++it) {
         float al[C], ga[C], de[C];
         {
             // w = dv / 4; r_i = D0_i - c0 (m_{i-1} + m_{i+1}) - b0 m_i + w_{i-1} T_{i-1} - w_{i+1} T_i,
@@ -418,6 +418,7 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
         // (6/h)(M m - H u): s_i + 2 m_i - 6 u_i - h2 (u_{i-1} - 2 u_i + u_{i+1}), the second
         // difference from the (nearly exact) first ones
         float dpH[C];
+        bool out;
         {
             q[0] = mp + m[0];
 #pragma unroll
@@ -433,9 +434,9 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
                 r[i] = d2f_bits(e);
                 dl = dr;
             }
-            helm_local_f<C, TP>(A.helf, r, dpH, sh);
+            out = helm_local_f<C, TP>(A.helf, r, dpH, sh);
         }
-        __syncthreads();                                             // B3
+        const int nan = __syncthreads_or(out);                       // B3
         if (t < 32) {
             CTab<float> const& T = A.helf;
             warp_solve_const<float, TP>(T, A.rhelf, fview(sh->hpd), fview(sh->hde), fview(sh->hE), fview(sh->hF));
@@ -444,7 +445,7 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
             const float mm = warp_max_bits((t < NW) ? fview(sh->wred[1])[t] : 0.0f);
             if (t == 0) {
                 int fl = 0;
-                if (!(dm < INFINITY) || !(mm < INFINITY) || sh->nan) fl = FLAG_NONFINITE;
+                if (!(dm < INFINITY) || !(mm < INFINITY) || nan) fl = FLAG_NONFINITE;
                 else if (dm <= A.tolf * fmaxf(1.0f, mm)) fl = FLAG_CONVERGED;
                 sh->flag = fl;
             }
@@ -462,7 +463,10 @@ __device__ __forceinline__ void sch_step_refined(const ModelArgs<double>& A, Shm
         }
         const int fl = sh->flag;
         if (fl & FLAG_CONVERGED) break;
-        bad = (fl & FLAG_NONFINITE) || it == A.max_iter;
+        if ((fl & FLAG_NONFINITE) || it == A.max_iter) {
+            bad = 1;
+            break;
+        }
     }
     if (bad) {
         Field<double, C> g = f;
